@@ -25,7 +25,9 @@ LIB = os.path.join(HERE, "libcosm.so")
 LIB_CHECKED = os.path.join(HERE, "libcosm_checked.so")
 BUILD = os.path.join(HERE, "_build")
 GENCODE = "arch=compute_103a,code=sm_103a"
-SOURCES = ["cosm_kernels.cu", "cosm_runtime.cu", "cosm_server.cu", "cosm_static.cu", "cosm_graph.cpp"]
+PATCH = ["cosm_patch_%s.cu" % f for f in ("f32_k2", "f16_k2", "f16_k4", "bf16_k2", "bf16_k4", "q16_k2", "q16_k4")]
+KERNELS = ["cosm_kernels.cu"] + PATCH  # units with device code that the checked build compiles apart
+SOURCES = KERNELS + ["cosm_runtime.cu", "cosm_server.cu", "cosm_static.cu", "cosm_graph.cpp"]
 
 
 def nvcc() -> str:
@@ -54,7 +56,7 @@ def build(force: bool = False, verbose: bool = False, checked: bool = False) -> 
     objs = []
     for src in SOURCES:
         # the checked library differs in the kernels only
-        tag = ".checked" if checked and src == "cosm_kernels.cu" else ""
+        tag = ".checked" if checked and src in KERNELS else ""
         obj = os.path.join(BUILD, src + tag + ".o")
         objs.append(obj)
         if not force and checked and not tag and os.path.exists(obj) and not _stale(obj):

@@ -11,6 +11,7 @@
 
 #include "../../include/cosm.h"
 #include "cosm_internal.h"
+#include "cosm_patch.h"
 
 #include <nvtx3/nvToolsExt.h>
 
@@ -89,6 +90,10 @@ struct cosm_handle {
     int mode = cosm::MODE_GENERAL_;       // kernel variant
     int32_t Q = 0, Wd = 0;          // 2D lattice geometry
     DevBuf<uint8_t> d_wnib;         // 2D lattice block weight bits
+    std::vector<uint8_t> nib;       // the same on the host
+    // 2D lattice kept in registers: weight words per patch, one table per
+    // shape, filled once when the shape is first chosen and then only read
+    DevBuf<uint32_t> d_pwt[cosm::kPatchShapes];
     bool fields = false;            // local fields given
     DevBuf<int32_t> d_h;            // local field per slot
     // per run
@@ -122,6 +127,9 @@ struct cosm_handle {
     // state of the last launch
     int replicas = 0;
     int K = 0, threads = 0, occupancy = 0, grid = 0;
+    int shape = -1;            // patch shape of the register kernels (-1: phases in shared memory)
+    bool ragged = false;       // the shape does not divide the lattice
+    int pgr = 0, pgc = 0, pfr = 0, pfc = 0;  // patch grid and its whole rows / columns of patches
     bool block_pairs = false;  // binary32 lattice tiles of two replicas: two 2x2 blocks per thread (even pass)
     bool staged = false;       // binary32 edge lists: colour records staged in shared memory
     size_t smem = 0;
@@ -139,6 +147,11 @@ struct cosm_handle {
 namespace cosm {
 
 int env_int(const char *name, int dflt);
+// The sweep kernel of a handle's layout: resident CTAs per SM (queue: as the
+// batch and serving launches run it), and its launches.
+int kernel_occupancy(const cosm_handle *h, int threads, size_t smem, bool queue);
+int kernel_launch(const LaunchCfg &cfg, const KernelArgs &a, cudaStream_t st);
+int kernel_launch_queue(const LaunchCfg &cfg, const BatchArgs &b, cudaStream_t st);
 // narrow_ties: among tiles keeping as many replicas resident, the narrower
 // one (more CTAs per SM) instead of the wider one on a full GPU.
 int choose_layout(cosm_handle *h, int replicas, bool narrow_ties = false);

@@ -49,6 +49,13 @@ struct InstView {
     const uint8_t *wnib;
     int32_t Q;
     int32_t Wd;
+    // lattices kept in registers: a grid of pgr x pgc patches of 2x2 blocks,
+    // one thread each; the first pfr rows (pfc columns) of patches are whole,
+    // the others one block shorter; pwt[k * pgr * pgc + patch] holds word k of
+    // a patch's weight bits (its own blocks, then the shifted ones)
+    const uint32_t *pwt;
+    int32_t pgr, pgc;
+    int32_t pfr, pfc;
     const float2 *alpha_tab;    // (alpha_s, dwt_step_s) for s = alpha_base ..
     int64_t alpha_base;
     int64_t S;            // sweeps of the trial (readout after sweep S)
@@ -146,6 +153,8 @@ struct LaunchCfg {
     int grid;      // CTAs
     size_t smem;   // dynamic shared bytes
     bool cooperative;
+    int shape = -1;   // lattices kept in registers: patch shape (cosm_patch.h), -1 otherwise
+    bool ragged = false;
 };
 
 // Shared-memory bytes for a tile and the resident CTAs per SM for a config.

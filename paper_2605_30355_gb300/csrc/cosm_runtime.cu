@@ -139,6 +139,7 @@ extern "C" void cosm_destroy(cosm_handle *h)
     h->d_segoff.release(); h->d_ready.release(); h->d_err.release(); h->d_best.release();
     h->d_spins.release();
     h->d_wnib.release();
+    for (auto &b : h->d_pwt) b.release();
     h->d_h.release(); h->d_energy.release(); h->d_bisB.release(); h->d_trace.release();
     h->d_bits.release(); h->d_qbuf.release(); h->d_delta.release(); h->d_items.release();
     delete h;
@@ -191,6 +192,7 @@ static int setup_lattice2d(cosm_handle *h)
     int rc = h->d_wnib.ensure(nib.size());
     if (rc) return rc;
     CK(cudaMemcpy(h->d_wnib.p, nib.data(), nib.size(), cudaMemcpyHostToDevice));
+    h->nib.swap(nib);
     h->Q = Q;
     h->Wd = Wd;
     h->mode = MODE_LATTICE2D_;
@@ -471,6 +473,184 @@ int cosm::env_int(const char *name, int dflt)
     return (s && *s) ? std::atoi(s) : dflt;
 }
 
+static int patch_call_for(int storage, int K, const PatchCall &c)
+{
+    const int none = c.what == PatchCall::OCCUPANCY ? 0 : -1;
+    switch (storage) {
+    case COSM_F32: return K == 2 ? patch_call_f32_k2(c) : none;
+    case COSM_F16: return K == 2 ? patch_call_f16_k2(c) : K == 4 ? patch_call_f16_k4(c) : none;
+    case COSM_BF16: return K == 2 ? patch_call_bf16_k2(c) : K == 4 ? patch_call_bf16_k4(c) : none;
+    default: return K == 2 ? patch_call_q16_k2(c) : K == 4 ? patch_call_q16_k4(c) : none;
+    }
+}
+
+static int patch_occupancy(int storage, int K, int shape, bool ragged, int threads, size_t smem)
+{
+    return patch_call_for(storage, K, PatchCall{PatchCall::OCCUPANCY, shape, ragged, threads, smem, 0, false, nullptr,
+                                                nullptr, nullptr});
+}
+
+int cosm::kernel_occupancy(const cosm_handle *h, int threads, size_t smem, bool queue)
+{
+    if (h->shape >= 0) return patch_occupancy(h->prm.storage, h->K, h->shape, h->ragged, threads, smem);
+    return queue ? batch_occupancy(h->prm.storage, h->K, h->mode, threads, smem)
+                 : sweep_occupancy(h->prm.storage, h->K, h->mode, threads, smem);
+}
+
+int cosm::kernel_launch(const LaunchCfg &cfg, const KernelArgs &a, cudaStream_t st)
+{
+    if (cfg.shape < 0) return sweep_launch(cfg, a, st);
+    return patch_call_for(cfg.storage, cfg.K, PatchCall{PatchCall::LAUNCH, cfg.shape, cfg.ragged, cfg.threads,
+                                                        cfg.smem, cfg.grid, cfg.cooperative, &a, nullptr, st});
+}
+
+int cosm::kernel_launch_queue(const LaunchCfg &cfg, const BatchArgs &b, cudaStream_t st)
+{
+    if (cfg.shape < 0) return batch_launch(cfg.storage, cfg.K, cfg.mode, cfg.grid, cfg.threads, cfg.smem, b, st);
+    return patch_call_for(cfg.storage, cfg.K, PatchCall{PatchCall::LAUNCH, cfg.shape, cfg.ragged, cfg.threads,
+                                                        cfg.smem, cfg.grid, false, nullptr, &b, st});
+}
+
+// How a side of B blocks splits into patches of at most P blocks: the grid,
+// and how many patches are whole (the others are one block shorter). False
+// when patches of P and P - 1 blocks cannot make up the side.
+static bool split_side(int B, int P, int *grid, int *whole)
+{
+    *grid = (B + P - 1) / P;
+    const int missing = *grid * P - B;
+    if (missing > *grid || (P == 1 && missing)) return false;
+    *whole = *grid - missing;
+    return true;
+}
+
+// Modelled SM cycles per sweep of a run in a patch layout: the instructions of
+// the warps that share an SM's schedulers at the issue rate the kernels
+// reach, or one CTA's latency where those do not fill it, times the waves of
+// tiles. Fitted to timings of 16 x 16 to 100 x 200 lattices, 32 to 2,048
+// replicas (within 15 %): binary32 100 x 100, 1,024 replicas, shapes 2x5 /
+// 2x4 / 2x3 / 2x2 measured 5.5 / 6.9 / 7.0 / 6.2 us per sweep, modelled 5.3 /
+// 6.9 / 7.1 / 5.6.
+static double patch_cost(int storage, int K, int R, int C, bool ragged, int warps, int occ, int replicas, int sms)
+{
+    const int NE = 2 * R + 2 * C - 1, words = K / 2;
+    // instructions per 2x2 block and pass, per warp, the twist and the wrap
+    // spread over their periods; instructions issued per scheduler and cycle
+    const double block = storage == COSM_F32 ? 42.0 : storage == COSM_Q16 ? 12.0 + 26.0 * words : 8.0 + 62.0 * words;
+    const double rate = storage == COSM_F32 ? 0.57 : storage == COSM_Q16 ? 0.62 : 0.60;
+    const double inst = 2.0 * R * C * block + 4.0 * NE + 30.0 + (ragged ? 4.0 * NE : 0.0);
+    const double tiles = std::ceil((double)replicas / K), slots = (double)occ * sms;
+    const double together = std::max(1.0, std::ceil(std::min(tiles, slots) / sms));
+    const double sweep = std::max(420.0 + 2.0 * inst, std::ceil(together * warps / 4.0) * inst / rate);
+    return sweep * std::max(1.0, tiles / slots);
+}
+
+// The same for 16-bit floats on shared memory, the least over tiles of two,
+// four and eight replicas (measured, 2x2 blocks per sweep and tile: 5.1 us for
+// 5,000 blocks and 0.64 us for 64 at two replicas, 4.2 us for 2,500 at four,
+// 8.2 us for 2,500 at eight). Binary32 and fixed point are faster in registers
+// wherever a shape fits; 16-bit floats, whose widening, wraps and rounding
+// outweigh the loads and stores saved, only up to about 100 x 100.
+static double shared_cost_16(int blocks, int replicas, int sms)
+{
+    const double per[3] = {1.9, 3.4, 6.6}, latency[3] = {1200.0, 1000.0, 1000.0};
+    double best = 1e300;
+    for (int k = 0; k < 3; ++k) {
+        const int K = 2 << k;
+        if ((size_t)blocks * 8 * K > 220 * 1024) continue;  // the tile does not fit
+        best = std::min(best, (per[k] * blocks + latency[k]) * std::max(1.0, std::ceil((double)replicas / K) / sms));
+    }
+    return best;
+}
+
+// Layout of a 2D lattice with its phases in registers (cosm_patch.cuh):
+// among the shapes and tile widths that fit, the one whose modelled time per
+// replica and sweep is lowest. Binary32 tiles hold two replicas, 16-bit ones
+// four or two. Returns false when no shape fits (the lattice then keeps its
+// phases in shared memory).
+static bool choose_patch(cosm_handle *h, int replicas, int forceK)
+{
+    const cosm_params &p = h->prm;
+    const int BR = h->Q / h->Wd, BC = h->Wd, only = env_int("COSM_PATCH", -2);
+    if (only == -1) return false;  // test hook: the shared-memory passes
+    const int Ks[2] = {p.storage == COSM_F32 ? 2 : 4, 2};
+    const bool f16 = p.storage == COSM_F16 || p.storage == COSM_BF16;
+    double best = f16 && only < 0 ? shared_cost_16(h->Q, replicas, h->num_sms) : 1e300;
+    for (int k = 0; k < (p.storage == COSM_F32 ? 1 : 2); ++k) {
+        const int K = Ks[k];
+        if (forceK && K != forceK) continue;
+        const size_t smem = sweep_smem_bytes(p.storage, K, h->g.n, p.n_bisectors, MODE_LATTICE2D_);
+        for (int s = 0; s < kPatchShapes; ++s) {
+            if (only >= 0 && s != only) continue;
+            // four 16-bit floats per site: patches above 2x2 blocks spill
+            if (only < 0 && f16 && K == 4 && kPatchR[s] * kPatchC[s] > 4) continue;
+            const int R = kPatchR[s], C = kPatchC[s], NE = 2 * R + 2 * C - 1;
+            int gr, gc, fr, fc;
+            if (!split_side(BR, R, &gr, &fr) || !split_side(BC, C, &gc, &fc)) continue;
+            // the published sites take the place of the tile
+            if ((int64_t)gr * gc * NE > h->g.n || gr * gc > 1024) continue;
+            const bool ragged = fr != gr || fc != gc;
+            const int T = (gr * gc + 31) / 32 * 32;
+            const int occ = patch_occupancy(p.storage, K, s, ragged, T, smem);
+            if (occ < 1) continue;
+            const double cost = patch_cost(p.storage, K, R, C, ragged, T / 32, occ, replicas, h->num_sms);
+            if (cost < best) {
+                best = cost;
+                h->shape = s;
+                h->ragged = ragged;
+                h->K = K;
+                h->threads = T;
+                h->occupancy = occ;
+                h->smem = smem;
+                h->pgr = gr;
+                h->pgc = gc;
+                h->pfr = fr;
+                h->pfc = fc;
+            }
+        }
+    }
+    return h->shape >= 0;
+}
+
+// Weight words of the chosen shape (InstView::pwt), from the block weight
+// bits: word k of a patch holds bits 32 k .. of its own blocks' nibbles, then
+// its shifted blocks'. In the float forms a pair across the torus seam takes
+// the negated step, so its weight bit is flipped (fixed point swaps the
+// roles instead).
+static int ensure_patch_weights(cosm_handle *h)
+{
+    DevBuf<uint32_t> &buf = h->d_pwt[h->shape];
+    if (buf.p) return COSM_OK;
+    const int R = kPatchR[h->shape], C = kPatchC[h->shape], T = h->pgr * h->pgc, words = (8 * R * C + 31) / 32;
+    const int BR = h->Q / h->Wd, BC = h->Wd;
+    const bool flip = h->prm.storage != COSM_Q16;
+    std::vector<uint32_t> wt((size_t)words * T, 0u);
+    for (int pr = 0; pr < h->pgr; ++pr) {
+        for (int pc = 0; pc < h->pgc; ++pc) {
+            const int r0 = pr * R - std::max(0, pr - h->pfr), nr = pr < h->pfr ? R : R - 1;
+            const int c0 = pc * C - std::max(0, pc - h->pfc), nc = pc < h->pfc ? C : C - 1;
+            for (int i = 0; i < nr; ++i) {
+                for (int j = 0; j < nc; ++j) {
+                    const int f = (r0 + i) * h->Wd + c0 + j;
+                    uint32_t odd = h->nib[(size_t)h->Q + f];
+                    if (flip && c0 + j == BC - 1) odd ^= 3u;
+                    if (flip && r0 + i == BR - 1) odd ^= 12u;
+                    const int b0 = 4 * (i * C + j), b1 = 4 * (R * C + i * C + j);
+                    const size_t t = (size_t)pr * h->pgc + pc;
+                    wt[(size_t)(b0 / 32) * T + t] |= (uint32_t)h->nib[(size_t)f] << (b0 % 32);
+                    wt[(size_t)(b1 / 32) * T + t] |= odd << (b1 % 32);
+                }
+            }
+        }
+    }
+    int rc = buf.ensure(wt.size());
+    if (rc) return rc;
+    if (cudaMemcpy(buf.p, wt.data(), wt.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess) {
+        buf.release();
+        return fail(COSM_ERR_CUDA, "copying the patch weights to the device failed");
+    }
+    return COSM_OK;
+}
+
 // Replicas per CTA (K) and threads per CTA: maximise resident replicas per
 // SM (COSM_K / COSM_THREADS override for experiments).
 int cosm::choose_layout(cosm_handle *h, int replicas, bool narrow_ties)
@@ -484,10 +664,22 @@ int cosm::choose_layout(cosm_handle *h, int replicas, bool narrow_ties)
     const int *Ks = p.storage == COSM_F32 ? Ks_f32 : Ks_f16;
     int forceK = env_int("COSM_K", 0), forceT = env_int("COSM_THREADS", 0);
     int bestK = 0, bestT = 0, bestOcc = 0;
+    // 2D lattices keep their phases in registers where a patch shape fits
+    // (forced threads and the cross-check switches take the passes on shared
+    // memory); else
     // binary32 lattice tiles of two replicas on an even number of block
     // columns take two adjacent 2x2 blocks per thread in the even pass
     // (COSM_SCALAR_F32 and COSM_SINGLE_BLOCKS keep the other passes
     // available as cross-checks)
+    h->shape = -1;
+    if (mode == MODE_LATTICE2D_ && !forceT && !std::getenv("COSM_SCALAR_F32") && !std::getenv("COSM_SINGLE_BLOCKS") &&
+        choose_patch(h, replicas, forceK)) {
+        h->block_pairs = false;
+        h->staged = false;
+        const size_t esz = p.storage == COSM_F32 ? 4 : 2;
+        h->tile_stride = (int64_t)(((size_t)h->g.n * h->K * esz + 15) / 16 * 16 / esz);
+        return ensure_patch_weights(h);
+    }
     const bool pairs_ok = mode == MODE_LATTICE2D_ && p.storage == COSM_F32 && h->Wd % 2 == 0 &&
                           !std::getenv("COSM_SCALAR_F32") && !std::getenv("COSM_SINGLE_BLOCKS");
     long bestScore = -1;
@@ -647,6 +839,13 @@ InstView cosm::inst_view(cosm_handle *h)
     v.wnib = h->d_wnib.p;
     v.Q = h->Q;
     v.Wd = h->Wd;
+    if (h->shape >= 0) {
+        v.pwt = h->d_pwt[h->shape].p;
+        v.pgr = h->pgr;
+        v.pgc = h->pgc;
+        v.pfr = h->pfr;
+        v.pfc = h->pfc;
+    }
     v.seed = h->seed;
     v.replicas = h->replicas;
     v.dwt_period = (h->prm.flags & COSM_NO_DWT) ? 0 : h->prm.dwt_period;
@@ -909,9 +1108,10 @@ static int run_range(cosm_handle *h, int64_t sweeps, int64_t s0, int64_t s1, int
     }
     a.segs = h->d_segs.p;
     a.seg_off = h->d_segoff.p;
-    LaunchCfg cfg{h->mode, h->prm.storage, h->K, h->threads, (int)(h->h_segoff.size() - 1), h->smem, waits};
+    LaunchCfg cfg{h->mode, h->prm.storage, h->K, h->threads, (int)(h->h_segoff.size() - 1), h->smem, waits,
+                  h->shape, h->ragged};
     h->grid = cfg.grid;
-    if (sweep_launch(cfg, a, st))
+    if (kernel_launch(cfg, a, st))
         return fail(COSM_ERR_CUDA, std::string("sweep launch: ") + cudaGetErrorString(cudaGetLastError()));
     h->launches = 1;
     h->stream = st;
@@ -1228,9 +1428,9 @@ static int launch_on_state(cosm_handle *h, int32_t flags, int64_t s0, int64_t s1
     a.v.S = s1;
     a.segs = h->d_segs.p;
     a.seg_off = h->d_segoff.p;
-    LaunchCfg cfg{h->mode, h->prm.storage, h->K, h->threads, (int)tiles, h->smem, false};
+    LaunchCfg cfg{h->mode, h->prm.storage, h->K, h->threads, (int)tiles, h->smem, false, h->shape, h->ragged};
     h->grid = cfg.grid;
-    if (sweep_launch(cfg, a, st))
+    if (kernel_launch(cfg, a, st))
         return fail(COSM_ERR_CUDA, std::string("sweep launch: ") + cudaGetErrorString(cudaGetLastError()));
     h->stream = st;
     return COSM_OK;
@@ -1326,6 +1526,8 @@ extern "C" int cosm_solve(const cosm_graph_desc *g, const cosm_params *p, int64_
 
 struct BatchClass {
     int storage, K, mode;
+    int shape;          // patch shape of lattices kept in registers (-1: none)
+    bool ragged;
     int threads;        // threads per CTA
     size_t smem;        // largest tile of the class
     int grid;           // CTAs (resident capacity, capped by units)
@@ -1448,7 +1650,7 @@ static int batch_instance_layout(cosm_batch *b, cosm_handle *h, int32_t replicas
     int rc;
     if (b->policy == 2) return choose_layout(h, replicas);
     if ((rc = choose_layout(h, 1 << 23, b->policy == 3))) return rc;
-    if (b->policy == 1 && h->K != (h->prm.storage == COSM_F32 ? 1 : 2)) {
+    if (b->policy == 1 && h->shape < 0 && h->K != (h->prm.storage == COSM_F32 ? 1 : 2)) {
         const int Kmin = h->prm.storage == COSM_F32 ? 1 : 2;
         const size_t esz = h->prm.storage == COSM_F32 ? 4 : 2;
         h->K = Kmin;
@@ -1476,7 +1678,7 @@ static int batch_layout(cosm_batch *b, const int64_t *sweeps, const int32_t *rep
             return fail(COSM_ERR_INVALID_ARG, "instance " + std::to_string(i) + ": bad sweeps or replicas");
         int rc;
         if ((rc = batch_instance_layout(b, h, replicas[i]))) return rc;
-        if (b->threads) {
+        if (b->threads && h->shape < 0) {
             h->threads = b->threads;
             while (h->threads > 64 && batch_occupancy(h->prm.storage, h->K, h->mode, h->threads, h->smem) == 0)
                 h->threads /= 2;
@@ -1498,17 +1700,18 @@ static int batch_layout(cosm_batch *b, const int64_t *sweeps, const int32_t *rep
     // shared memory); their units form one queue, longest trials first
     b->classes.clear();
     b->h_units.clear();
-    struct Key { int storage, K, mode, threads, occ; };
+    struct Key { int storage, K, mode, shape; bool ragged; int threads, occ; };
     std::vector<Key> keys;
     std::vector<int> cls((size_t)n);
     for (int i = 0; i < n; ++i) {
         const cosm_handle *h = b->hs[(size_t)i];
-        const Key k{h->prm.storage, h->K, h->mode, h->threads,
-                    batch_occupancy(h->prm.storage, h->K, h->mode, h->threads, h->smem)};
+        const Key k{h->prm.storage, h->K, h->mode, h->shape, h->shape >= 0 && h->ragged, h->threads,
+                    kernel_occupancy(h, h->threads, h->smem, true)};
         int c = -1;
         for (size_t q = 0; q < keys.size() && c < 0; ++q) {
             const Key &o = keys[q];
-            if (o.storage == k.storage && o.K == k.K && o.mode == k.mode && o.threads == k.threads && o.occ == k.occ)
+            if (o.storage == k.storage && o.K == k.K && o.mode == k.mode && o.shape == k.shape && o.ragged == k.ragged &&
+                o.threads == k.threads && o.occ == k.occ)
                 c = (int)q;
         }
         if (c < 0) {
@@ -1519,7 +1722,7 @@ static int batch_layout(cosm_batch *b, const int64_t *sweeps, const int32_t *rep
     }
     int dev_sms = b->hs[0]->num_sms;
     for (size_t c = 0; c < keys.size(); ++c) {
-        BatchClass bc{keys[c].storage, keys[c].K, keys[c].mode, keys[c].threads, 0, 0,
+        BatchClass bc{keys[c].storage, keys[c].K, keys[c].mode, keys[c].shape, keys[c].ragged, keys[c].threads, 0, 0,
                       (int32_t)b->h_units.size(), 0};
         std::vector<std::pair<double, BatchUnit>> us;
         for (int i = 0; i < n; ++i) {
@@ -1535,10 +1738,14 @@ static int batch_layout(cosm_batch *b, const int64_t *sweeps, const int32_t *rep
         for (auto &u : us) b->h_units.push_back(u.second);
         bc.units = (int32_t)us.size();
         int T = bc.threads;
-        int occ = batch_occupancy(bc.storage, bc.K, bc.mode, T, bc.smem);
-        while (occ == 0 && T > 64) {
+        const auto occ_of = [&](int threads) {
+            return bc.shape >= 0 ? patch_occupancy(bc.storage, bc.K, bc.shape, bc.ragged, threads, bc.smem)
+                                 : batch_occupancy(bc.storage, bc.K, bc.mode, threads, bc.smem);
+        };
+        int occ = occ_of(T);
+        while (occ == 0 && T > 64 && bc.shape < 0) {
             T /= 2;
-            occ = batch_occupancy(bc.storage, bc.K, bc.mode, T, bc.smem);
+            occ = occ_of(T);
         }
         if (occ == 0) return fail(COSM_ERR_TOO_LARGE, "a batch tile does not fit on an SM");
         bc.threads = T;
@@ -1577,7 +1784,8 @@ static int batch_enqueue(cosm_batch *b, cudaStream_t st)
         const BatchClass &bc = b->classes[c];
         CK(cudaStreamWaitEvent(b->side[c], b->ev[0], 0));
         BatchArgs a{b->d_insts.p, b->d_units.p + bc.unit0, bc.units, b->d_counters.p + c};
-        if (bc.units > 0 && batch_launch(bc.storage, bc.K, bc.mode, bc.grid, bc.threads, bc.smem, a, b->side[c]))
+        if (bc.units > 0 && kernel_launch_queue(LaunchCfg{bc.mode, bc.storage, bc.K, bc.threads, bc.grid, bc.smem, false, bc.shape,
+                                                       bc.ragged}, a, b->side[c]))
             return fail(COSM_ERR_CUDA, std::string("batch launch: ") + cudaGetErrorString(cudaGetLastError()));
         CK(cudaEventRecord(b->ev[c + 1], b->side[c]));
     }
@@ -1608,6 +1816,7 @@ extern "C" int cosm_batch_run(cosm_batch *b, const int64_t *sweeps, const int32_
     sig.push_back((int64_t)(uintptr_t)b->d_counters.p);
     for (const BatchClass &bc : b->classes) {
         sig.push_back(bc.storage); sig.push_back(bc.K); sig.push_back(bc.mode); sig.push_back(bc.threads);
+        sig.push_back(bc.shape); sig.push_back(bc.ragged);
         sig.push_back((int64_t)bc.smem); sig.push_back(bc.grid); sig.push_back(bc.unit0); sig.push_back(bc.units);
     }
     if (!b->exec || sig != b->sig) {

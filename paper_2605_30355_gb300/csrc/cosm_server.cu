@@ -80,6 +80,10 @@ struct cosm_server {
     DevBuf<InstView> d_insts;
     DevBuf<BatchUnit> d_units;
     DevBuf<int32_t> d_counters;
+    // classes after the first run on side streams forked from st, so that a
+    // class of few tiles does not hold up the next one
+    std::vector<cudaStream_t> side;
+    std::vector<cudaEvent_t> ev;  // fork, then one per side stream
     std::thread worker;
 
     double now() const
@@ -141,11 +145,12 @@ static int run_chunk(cosm_server *s, const std::vector<Request *> &act)
 {
     const int n = (int)act.size();
     std::vector<InstView> views((size_t)n);
-    struct Key { int storage, K, mode; };
+    struct Key { int storage, K, mode, shape; bool ragged; int threads; };  // threads: of the patch shape
     std::vector<Key> keys;
     std::vector<std::vector<BatchUnit>> per;
     std::vector<size_t> smem;
     std::vector<int> max_ec;
+    std::vector<cosm_handle *> rep;  // one handle of each class
     for (int i = 0; i < n; ++i) {
         Request *r = act[(size_t)i];
         cosm_handle *h = r->h;
@@ -156,13 +161,18 @@ static int run_chunk(cosm_server *s, const std::vector<Request *> &act)
         v.S = r->S;
         views[(size_t)i] = v;
         int c = -1;
+        const Key own{h->prm.storage, h->K, h->mode, h->shape, h->shape >= 0 && h->ragged,
+                      h->shape >= 0 ? h->threads : 0};
         for (size_t k = 0; k < keys.size(); ++k)
-            if (keys[k].storage == h->prm.storage && keys[k].K == h->K && keys[k].mode == h->mode) c = (int)k;
+            if (keys[k].storage == own.storage && keys[k].K == own.K && keys[k].mode == own.mode &&
+                keys[k].shape == own.shape && keys[k].ragged == own.ragged && keys[k].threads == own.threads)
+                c = (int)k;
         if (c < 0) {
-            keys.push_back(Key{h->prm.storage, h->K, h->mode});
+            keys.push_back(own);
             per.emplace_back();
             smem.push_back(0);
             max_ec.push_back(0);
+            rep.push_back(h);
             c = (int)keys.size() - 1;
         }
         smem[(size_t)c] = std::max(smem[(size_t)c], h->smem);
@@ -185,21 +195,41 @@ static int run_chunk(cosm_server *s, const std::vector<Request *> &act)
     CK(cudaMemcpyAsync(s->d_insts.p, views.data(), views.size() * sizeof(InstView), cudaMemcpyHostToDevice, s->st));
     CK(cudaMemcpyAsync(s->d_units.p, units.data(), units.size() * sizeof(BatchUnit), cudaMemcpyHostToDevice, s->st));
     CK(cudaMemsetAsync(s->d_counters.p, 0, keys.size() * 4, s->st));
+    while (s->side.size() + 1 < keys.size()) {
+        cudaStream_t st;
+        CK(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
+        s->side.push_back(st);
+    }
+    while (s->ev.size() < keys.size()) {
+        cudaEvent_t e;
+        CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+        s->ev.push_back(e);
+    }
+    if (keys.size() > 1) CK(cudaEventRecord(s->ev[0], s->st));
     for (size_t c = 0; c < keys.size(); ++c) {
-        int T = s->cfg.threads ? s->cfg.threads : std::min(512, std::max(64, ((max_ec[c] + 1) / 2 + 31) / 32 * 32));
-        int occ = batch_occupancy(keys[c].storage, keys[c].K, keys[c].mode, T, smem[c]);
-        while (occ == 0 && T > 64) {
+        // a patch shape has its own thread count
+        int T = keys[c].threads ? keys[c].threads
+                : s->cfg.threads ? s->cfg.threads
+                                 : std::min(512, std::max(64, ((max_ec[c] + 1) / 2 + 31) / 32 * 32));
+        cosm_handle *h = rep[c];
+        int occ = kernel_occupancy(h, T, smem[c], true);
+        while (occ == 0 && T > 64 && !keys[c].threads) {
             T /= 2;
-            occ = batch_occupancy(keys[c].storage, keys[c].K, keys[c].mode, T, smem[c]);
+            occ = kernel_occupancy(h, T, smem[c], true);
         }
         if (occ == 0) return fail(COSM_ERR_TOO_LARGE, "a serving tile does not fit on an SM");
         const int32_t cnt = (int32_t)per[c].size();
         const int grid = (int)std::min<int64_t>((int64_t)occ * s->num_sms, cnt);
         BatchArgs a{s->d_insts.p, s->d_units.p + unit0[c], cnt, s->d_counters.p + c};
-        if (batch_launch(keys[c].storage, keys[c].K, keys[c].mode, grid, T, smem[c], a, s->st))
+        cudaStream_t st = c ? s->side[c - 1] : s->st;
+        if (c > 0) CK(cudaStreamWaitEvent(st, s->ev[0], 0));
+        if (kernel_launch_queue(LaunchCfg{keys[c].mode, keys[c].storage, keys[c].K, T, grid, smem[c], false,
+                                          keys[c].shape, keys[c].ragged}, a, st))
             return fail(COSM_ERR_CUDA, std::string("serving launch: ") + cudaGetErrorString(cudaGetLastError()));
         s->launches++;
+        if (c > 0) CK(cudaEventRecord(s->ev[c], st));
     }
+    for (size_t c = 1; c < keys.size(); ++c) CK(cudaStreamWaitEvent(s->st, s->ev[c], 0));
     CK(cudaStreamSynchronize(s->st));
     return COSM_OK;
 }
@@ -249,6 +279,8 @@ static void worker_main(cosm_server *s)
             NvtxRange range("cosm_server_chunk");
             rc = run_chunk(s, act);
         }
+        if (rc)  // classes launched before the failure end before their requests go
+            for (cudaStream_t q : s->side) cudaStreamSynchronize(q);
         std::vector<Request *> keep;
         for (Request *r : act) {
             if (rc) {
@@ -355,6 +387,8 @@ extern "C" void cosm_server_destroy(cosm_server *s)
     s->d_insts.release();
     s->d_units.release();
     s->d_counters.release();
+    for (cudaStream_t q : s->side) cudaStreamDestroy(q);
+    for (cudaEvent_t e : s->ev) cudaEventDestroy(e);
     if (s->st) cudaStreamDestroy(s->st);
     delete s;
 }
