@@ -26,7 +26,8 @@ LIB_CHECKED = os.path.join(HERE, "libcosm_checked.so")
 BUILD = os.path.join(HERE, "_build")
 GENCODE = "arch=compute_103a,code=sm_103a"
 PATCH = ["cosm_patch_%s.cu" % f for f in ("f32_k2", "f16_k2", "f16_k4", "bf16_k2", "bf16_k4", "q16_k2", "q16_k4")]
-KERNELS = ["cosm_kernels.cu"] + PATCH  # units with device code that the checked build compiles apart
+EDGES = ["cosm_edges_%s.cu" % f for f in ("f32", "f16", "bf16", "q16")]
+KERNELS = ["cosm_kernels.cu"] + EDGES + PATCH  # units with device code that the checked build compiles apart
 SOURCES = KERNELS + ["cosm_runtime.cu", "cosm_server.cu", "cosm_static.cu", "cosm_graph.cpp"]
 
 

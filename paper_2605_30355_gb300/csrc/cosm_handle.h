@@ -6,11 +6,13 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <memory>
 #include <string>
 #include <vector>
 
 #include "../../include/cosm.h"
 #include "cosm_internal.h"
+#include "cosm_edges.h"
 #include "cosm_patch.h"
 
 #include <nvtx3/nvToolsExt.h>
@@ -66,6 +68,20 @@ struct DevBuf {
     }
 };
 
+// A sweep's edges laid out for one tile width and thread count
+// (cosm_edges.h); only read once it is filled.
+struct RecordTable {
+    int K = 0, threads = 0, format = -1, n_colours = 0;
+    DevBuf<uint32_t> rec, counts;
+    DevBuf<int32_t> starts;
+    void release()
+    {
+        rec.release();
+        counts.release();
+        starts.release();
+    }
+};
+
 }  // namespace cosm
 
 struct cosm_handle {
@@ -77,6 +93,7 @@ struct cosm_handle {
     int num_sms = 0;
     bool lattice = false;
     int64_t W = 0;                  // total weight
+    int32_t wmax = 0;               // largest |w|
     int64_t wbound = 0;             // sum over colours of the largest |w|, plus the largest |h|
     std::vector<int32_t> slot_of;   // original id -> slot
     std::vector<int32_t> orig_of;   // slot -> original id
@@ -85,6 +102,11 @@ struct cosm_handle {
     DevBuf<uint32_t> d_ij;
     DevBuf<int8_t> d_w;
     DevBuf<uint32_t> d_ijs;         // +-1 weights on <= 2^15 slots: records with the sign in bit 31
+    std::vector<uint32_t> h_ij;     // colour-major records and weights on the host
+    std::vector<int8_t> h_wv;
+    std::vector<std::unique_ptr<cosm::RecordTable>> tables;
+    const cosm::RecordTable *table = nullptr;  // the current layout's
+    int format = -1;                // record-table format of the current layout (-1: none)
     DevBuf<int32_t> d_orig;
     DevBuf<int32_t> d_off;          // colour offsets
     int mode = cosm::MODE_GENERAL_;       // kernel variant
@@ -155,6 +177,10 @@ int kernel_launch_queue(const LaunchCfg &cfg, const BatchArgs &b, cudaStream_t s
 // narrow_ties: among tiles keeping as many replicas resident, the narrower
 // one (more CTAs per SM) instead of the wider one on a full GPU.
 int choose_layout(cosm_handle *h, int replicas, bool narrow_ties = false);
+// Half a thread count, in whole warps where the kernel needs them.
+inline int half_threads(int threads, bool warps) { return warps ? std::max(32, threads / 64 * 32) : threads / 2; }
+// The device tables of the chosen layout (h->K, h->threads, h->shape).
+int ensure_tables(cosm_handle *h);
 int ensure_run_buffers(cosm_handle *h, int replicas);
 InstView inst_view(cosm_handle *h);
 int upload_alpha(cosm_handle *h, int64_t S, cudaStream_t st);

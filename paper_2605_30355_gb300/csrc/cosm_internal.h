@@ -42,6 +42,12 @@ struct InstView {
     // in bit 0 ([w = -1] | slot(src) << 1 | slot(dst) << 16), so the
     // binary32 edge-list sweep loads one word per edge; nullptr otherwise
     const uint32_t *ijs;
+    // the same edges as a record table for this launch's tile width and thread
+    // count (cosm_edges.h): n_colours non-empty colours
+    const uint32_t *rec;
+    const uint32_t *counts;
+    const int32_t *starts;
+    int32_t n_colours;
     const int32_t *orig_of;  // slot -> original vertex id (Philox init key)
     // 2D lattice mode: Q = n/4 slots per sublattice, Wd = L2/2 columns;
     // wnib[pass * Q + f] holds the weight bits of the four edges of 2x2
@@ -155,6 +161,7 @@ struct LaunchCfg {
     bool cooperative;
     int shape = -1;   // lattices kept in registers: patch shape (cosm_patch.h), -1 otherwise
     bool ragged = false;
+    int format = -1;  // edge lists from record tables: their format (cosm_edges.h), -1 otherwise
 };
 
 // Shared-memory bytes for a tile and the resident CTAs per SM for a config.

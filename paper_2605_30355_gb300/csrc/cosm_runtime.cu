@@ -140,6 +140,7 @@ extern "C" void cosm_destroy(cosm_handle *h)
     h->d_spins.release();
     h->d_wnib.release();
     for (auto &b : h->d_pwt) b.release();
+    for (auto &t : h->tables) t->release();
     h->d_h.release(); h->d_energy.release(); h->d_bisB.release(); h->d_trace.release();
     h->d_bits.release(); h->d_qbuf.release(); h->d_delta.release(); h->d_items.release();
     delete h;
@@ -377,6 +378,12 @@ extern "C" int cosm_create(const cosm_graph_desc *gd, const cosm_params *p, cosm
         if (g.color[(size_t)a] != g.color[(size_t)b]) return g.color[(size_t)a] < g.color[(size_t)b];
         return h->slot_of[(size_t)g.src[(size_t)a]] < h->slot_of[(size_t)g.src[(size_t)b]];
     });
+    // instances that never take record tables (whose rows are arranged for
+    // their own tile width) have their colours' edges ordered here
+    int32_t wmax = 0;
+    for (int64_t e = 0; e < g.m; ++e) wmax = std::max(wmax, std::abs(g.w[(size_t)e]));
+    const bool plain = (p->flags & COSM_NO_SCS) || (p->storage != COSM_Q16 && wmax > 63) ||
+                       std::getenv("COSM_STAGE") || std::getenv("COSM_SPLIT_W");
     {
         std::vector<int32_t> ss((size_t)g.m), ds((size_t)g.m);
         for (int64_t e = 0; e < g.m; ++e) {
@@ -387,7 +394,7 @@ extern "C" int cosm_create(const cosm_graph_desc *gd, const cosm_params *p, cosm
         while (a < g.m) {
             int64_t z = a;
             while (z < g.m && g.color[(size_t)order[(size_t)z]] == g.color[(size_t)order[(size_t)a]]) ++z;
-            if (!std::getenv("COSM_SRC_ORDER")) balance_banks(order.data() + a, z - a, ss, ds);
+            if (plain && !std::getenv("COSM_SRC_ORDER")) balance_banks(order.data() + a, z - a, ss, ds);
             a = z;
         }
     }
@@ -403,6 +410,9 @@ extern "C" int cosm_create(const cosm_graph_desc *gd, const cosm_params *p, cosm
         h->W += g.w[(size_t)e];
     }
     for (int c = 0; c < h->C; ++c) h->off[c + 1] += h->off[c];
+    h->wmax = wmax;
+    h->h_ij = ij;
+    h->h_wv = wv;
     h->wbound = std::min(colour_weight_bound(h->off, h->C, wv.data(), gd->h, g.n),
                          vertex_weight_bound(g.n, g.m, g.src.data(), g.dst.data(), g.w.data(), gd->h));
     // device copies
@@ -490,8 +500,25 @@ static int patch_occupancy(int storage, int K, int shape, bool ragged, int threa
                                                 nullptr, nullptr});
 }
 
+static int edges_call_for(int storage, const EdgesCall &c)
+{
+    switch (storage) {
+    case COSM_F32: return edges_call_f32(c);
+    case COSM_F16: return edges_call_f16(c);
+    case COSM_BF16: return edges_call_bf16(c);
+    default: return edges_call_q16(c);
+    }
+}
+
+static int edges_occupancy(int storage, int K, int format, int threads, size_t smem)
+{
+    return edges_call_for(storage, EdgesCall{EdgesCall::OCCUPANCY, K, format, threads, smem, 0, false, nullptr, nullptr,
+                                             nullptr});
+}
+
 int cosm::kernel_occupancy(const cosm_handle *h, int threads, size_t smem, bool queue)
 {
+    if (h->format >= 0) return edges_occupancy(h->prm.storage, h->K, h->format, threads, smem);
     if (h->shape >= 0) return patch_occupancy(h->prm.storage, h->K, h->shape, h->ragged, threads, smem);
     return queue ? batch_occupancy(h->prm.storage, h->K, h->mode, threads, smem)
                  : sweep_occupancy(h->prm.storage, h->K, h->mode, threads, smem);
@@ -499,6 +526,9 @@ int cosm::kernel_occupancy(const cosm_handle *h, int threads, size_t smem, bool 
 
 int cosm::kernel_launch(const LaunchCfg &cfg, const KernelArgs &a, cudaStream_t st)
 {
+    if (cfg.format >= 0)
+        return edges_call_for(cfg.storage, EdgesCall{EdgesCall::LAUNCH, cfg.K, cfg.format, cfg.threads, cfg.smem,
+                                                     cfg.grid, cfg.cooperative, &a, nullptr, st});
     if (cfg.shape < 0) return sweep_launch(cfg, a, st);
     return patch_call_for(cfg.storage, cfg.K, PatchCall{PatchCall::LAUNCH, cfg.shape, cfg.ragged, cfg.threads,
                                                         cfg.smem, cfg.grid, cfg.cooperative, &a, nullptr, st});
@@ -506,6 +536,9 @@ int cosm::kernel_launch(const LaunchCfg &cfg, const KernelArgs &a, cudaStream_t 
 
 int cosm::kernel_launch_queue(const LaunchCfg &cfg, const BatchArgs &b, cudaStream_t st)
 {
+    if (cfg.format >= 0)
+        return edges_call_for(cfg.storage, EdgesCall{EdgesCall::LAUNCH, cfg.K, cfg.format, cfg.threads, cfg.smem,
+                                                     cfg.grid, false, nullptr, &b, st});
     if (cfg.shape < 0) return batch_launch(cfg.storage, cfg.K, cfg.mode, cfg.grid, cfg.threads, cfg.smem, b, st);
     return patch_call_for(cfg.storage, cfg.K, PatchCall{PatchCall::LAUNCH, cfg.shape, cfg.ragged, cfg.threads,
                                                         cfg.smem, cfg.grid, false, nullptr, &b, st});
@@ -651,6 +684,250 @@ static int ensure_patch_weights(cosm_handle *h)
     return COSM_OK;
 }
 
+// Format of the record tables of an edge-list instance with tiles of K
+// replicas, -1 where it takes the plain records: the simultaneous update,
+// staged or split records (test hooks), thread counts that are not whole
+// warps, and float weights of 64 and more, whose bits do not fit.
+static int record_format(const cosm_handle *h, int K)
+{
+    const cosm_params &p = h->prm;
+    if (h->mode != MODE_GENERAL_ || std::getenv("COSM_STAGE") || std::getenv("COSM_SPLIT_W") ||
+        env_int("COSM_THREADS", 0) % 32)
+        return -1;
+    const int E = K * (p.storage == COSM_F32 ? 4 : 2);
+    const bool each = p.storage == COSM_F32 && wrap_period(p.alpha0_deg, p.dwt_ratio, p.dwt_period, p.flags, h->mode,
+                                                           p.storage, h->wbound) == 0;
+    if (h->d_ijs.p && !each) return EDGES_SIGN;
+    const int more = each ? EDGES_EACH : 0;
+    // one word (half the record traffic of a weighted graph) where it holds
+    if (E >= 8 && h->g.n <= (1 << 14) && h->wmax <= (E == 8 ? 3 : 7)) return EDGES_PACK | more;
+    if (p.storage != COSM_Q16 && h->wmax > 63) return -1;
+    return EDGES_WEIGHT | more;
+}
+
+// Modelled SM cycles per sweep of a run of edge-list tiles of K replicas with T
+// threads (record tables): what the CTAs that share an SM issue and move
+// through shared memory, plus part of one CTA's latency per sweep (which more
+// CTAs hide), times the waves of tiles. Fitted to random 3-regular graphs of
+// 20,000 vertices, G(n, m) graphs of 2,000 and 10,000 and 3D lattices of 1,728
+// and 21,952, 32 to 2,048 replicas: within 20 %, e.g. G(9973, 24931) with
+// weights to 3 at two replicas per tile and 256 / 512 / 1,024 threads 22.3 /
+// 24.1 / 33.7 us per sweep of 1,024 replicas, modelled 23.4 / 24.9 / 33.
+static double edges_cost(const cosm_handle *h, int K, int format, int T, int occ, int replicas)
+{
+    const int st = h->prm.storage, W = T / 32, E = K * (st == COSM_F32 ? 4 : 2);
+    const double words = K / 2.0, colours = h->C;
+    // instructions and shared-memory wavefronts of a row of 32 edges
+    double inst = st == COSM_F32 ? 12.0 + 9.0 * std::max(1.0, words)
+                                 : st == COSM_Q16 ? 14.0 + 6.5 * words : 12.0 + 19.0 * words;
+    if ((format & ~EDGES_EACH) != EDGES_SIGN) inst += 2.0;
+    if (format >= 0 && (format & EDGES_EACH)) inst += 6.0 * std::max(1.0, words);
+    const double waves = (E == 4 ? 5.2 : E == 8 ? 9.0 : 17.8) + ((format & ~EDGES_EACH) == EDGES_WEIGHT ? 2.6 : 1.5);
+    double rows = 0.0, steps = 0.0;  // rows of all colours, and of the busiest warp
+    for (int c = 0; c < h->C; ++c) {
+        const int r = (h->off[c + 1] - h->off[c] + 31) / 32;
+        rows += r;
+        steps += (r + W - 1) / W;
+    }
+    // the twist and the wrap after the colours, every second sweep or so, and a field pass
+    const double slots = h->g.n / 32.0, passes = 0.5 + (h->fields ? 1.0 : 0.0);
+    const double tiles = std::ceil((double)replicas / K), room = (double)occ * h->num_sms;
+    const double r = std::max(1.0, std::ceil(std::min(tiles, room) / h->num_sms));
+    const double rate = std::min(2.4, 0.15 * r * W);  // instructions per SM and cycle
+    const double issue = (rows * inst + W * colours * 40.0 + slots * passes * (6.0 + 6.0 * std::max(1.0, words))) / rate;
+    const double move = (rows * waves + slots * passes * E / 2.0) / 0.8;
+    const double latency = colours * 250.0 + steps * (E >= 16 ? 70.0 : 110.0) + slots / W * passes * 60.0;
+    return (r * std::max(issue, move) + 0.6 * latency / r) * std::max(1.0, tiles / room);
+}
+
+// Tile width and threads of an edge-list instance on record tables. False
+// when no width and thread count take them.
+static bool choose_edges(cosm_handle *h, int replicas, int forceK, int forceT)
+{
+    const cosm_params &p = h->prm;
+    const int Ts[8] = {64, 128, 192, 256, 384, 512, 768, 1024};
+    double best = 1e300;
+    for (int K = p.storage == COSM_F32 ? 1 : 2; K <= (p.storage == COSM_F32 ? 4 : 8); K *= 2) {
+        if (forceK && K != forceK) continue;
+        const int format = record_format(h, K);
+        if (format < 0) return false;
+        const size_t smem = sweep_smem_bytes(p.storage, K, h->g.n, p.n_bisectors, h->mode);
+        for (int k = 0; k < (forceT ? 1 : 8); ++k) {
+            const int T = forceT ? forceT : Ts[k];
+            const int occ = edges_occupancy(p.storage, K, format, T, smem);
+            if (occ < 1) continue;
+            const double cost = edges_cost(h, K, format, T, occ, replicas);
+            if (cost < best) {
+                best = cost;
+                h->K = K;
+                h->threads = T;
+                h->occupancy = occ;
+                h->smem = smem;
+                h->format = format;
+            }
+        }
+    }
+    return best < 1e300;
+}
+
+// Order of one colour's edges e0 .. e1 - 1 in the rows of a table. A phase
+// access of 4, 8 or 16 bytes per lane takes one wavefront per 32, 16 or 8
+// lanes when their slots are distinct modulo R = 128 / E, so the edges are
+// dealt in groups of R with distinct source residues and, as far as they go
+// round, distinct destination residues: each source residue gives an edge
+// whose destination residue is still free, both rotated from group to group;
+// places left over take the fullest cells. Edges of one colour share no
+// vertex, so the order changes no result. Extra wavefronts of 7,500 random
+// edges: 7 / 19 / 41 % for R = 8 / 16 / 32 (161 / 206 / 251 % unarranged), at
+// 16 ns an edge.
+static void arrange_rows(const uint32_t *ij, int e0, int e1, int R, std::vector<int32_t> &out)
+{
+    const int cnt = e1 - e0;
+    out.resize((size_t)cnt);
+    if (cnt <= R || std::getenv("COSM_SRC_ORDER")) {
+        for (int k = 0; k < cnt; ++k) out[(size_t)k] = e0 + k;
+        return;
+    }
+    std::vector<int32_t> head((size_t)R * R, -1), next((size_t)cnt);
+    uint32_t mask[32] = {0};  // destination residues a source residue still has
+    int rows[32] = {0}, cols[32] = {0};
+    for (int k = cnt - 1; k >= 0; --k) {
+        const int a = (int)(ij[e0 + k] & 0xFFFFu) % R, b = (int)(ij[e0 + k] >> 16) % R;
+        next[(size_t)k] = head[(size_t)(a * R + b)];
+        head[(size_t)(a * R + b)] = k;
+        mask[a] |= 1u << b;
+        ++rows[a];
+        ++cols[b];
+    }
+    int done = 0;
+    auto take = [&](int a, int b) {
+        int32_t &hd = head[(size_t)(a * R + b)];
+        out[(size_t)done++] = e0 + hd;
+        hd = next[(size_t)hd];
+        if (hd < 0) mask[a] &= ~(1u << b);
+        --rows[a];
+        --cols[b];
+    };
+    const uint32_t full = R == 32 ? 0xFFFFFFFFu : (1u << R) - 1;
+    for (int g = 0; done < cnt; ++g) {
+        uint32_t used = 0;
+        const int stop = std::min(cnt, done + R);
+        for (int i = 0; i < R && done < stop; ++i) {
+            const int a = (i + g) % R, s = (a + g) % R;
+            const uint32_t open = mask[a] & ~used;
+            if (!open) continue;
+            const uint32_t turned = ((open >> s) | (s ? open << (R - s) : 0u)) & full;
+            const int b = (__builtin_ctz(turned) + s) % R;
+            used |= 1u << b;
+            take(a, b);
+        }
+        while (done < stop) {
+            int a = 0, b = -1;
+            for (int i = 1; i < R; ++i)
+                if (rows[i] > rows[a]) a = i;
+            for (uint32_t m = mask[a]; m; m &= m - 1) {
+                const int q = __builtin_ctz(m);
+                if (b < 0 || cols[q] > cols[b]) b = q;
+            }
+            take(a, b);
+        }
+    }
+}
+
+// Builds the record table of the current layout (cosm_edges.h).
+static int ensure_records(cosm_handle *h)
+{
+    for (const auto &t : h->tables) {
+        if (t->K == h->K && t->threads == h->threads && t->format == h->format) {
+            h->table = t.get();
+            return COSM_OK;
+        }
+    }
+    if (h->threads < 32 || h->threads % 32) return fail(COSM_ERR_INVALID_ARG, "record tables need whole warps");
+    const int fmt = h->format & ~EDGES_EACH, W = h->threads / 32, RW = fmt == EDGES_WEIGHT ? 2 : 1;
+    const uint32_t E = (uint32_t)(h->K * (h->prm.storage == COSM_F32 ? 4 : 2));
+    const bool q16 = h->prm.storage == COSM_Q16;
+    int nc = 0;
+    for (int c = 0; c < h->C; ++c) nc += h->off[c + 1] > h->off[c];  // an empty colour needs no barrier
+    std::vector<uint32_t> counts((size_t)W * (nc + 1), 0u);
+    std::vector<int32_t> starts((size_t)W + 1, 0), at((size_t)W);
+    for (int c = 0, k = 0; c < h->C; ++c) {
+        const int ec = h->off[c + 1] - h->off[c], rows = (ec + 31) / 32;
+        if (!rows) continue;
+        for (int w = 0; w < W; ++w) {
+            const int mine = rows / W + (w < rows % W);
+            counts[(size_t)w * (nc + 1) + k] = (uint32_t)mine | (ec % 32 && (rows - 1) % W == w ? kPartial : 0u);
+            starts[(size_t)w + 1] += mine * 32 * RW;
+        }
+        ++k;
+    }
+    for (int w = 0; w < W; ++w) {
+        counts[(size_t)w * (nc + 1) + nc] = counts[(size_t)w * (nc + 1)];
+        starts[(size_t)w + 1] += starts[(size_t)w] + kRowsAhead * 32 * RW;
+    }
+    std::vector<uint32_t> rec((size_t)starts[(size_t)W], kNoEdge);
+    std::copy(starts.begin(), starts.end() - 1, at.begin());
+    std::vector<int32_t> order;
+    for (int c = 0; c < h->C; ++c) {
+        const int ec = h->off[c + 1] - h->off[c];
+        arrange_rows(h->h_ij.data(), h->off[c], h->off[c + 1], (int)(128 / E), order);
+        for (int k = 0; k < ec; ++k) {
+            const int e = order[(size_t)k], lane = k % 32, w = k / 32 % W;
+            uint32_t *r = rec.data() + at[(size_t)w] + lane * RW;
+            const uint32_t si = h->h_ij[(size_t)e] & 0xFFFFu, sj = h->h_ij[(size_t)e] >> 16;
+            const int wt = h->h_wv[(size_t)e];
+            if (fmt == EDGES_SIGN) {
+                r[0] = (wt < 0 ? 1u : 0u) | (si << 1) | (sj << 16);
+            } else if (fmt == EDGES_PACK) {
+                r[0] = (uint32_t)(wt + (int)E / 2) | si * E | (sj << 18);
+            } else {
+                uint32_t bits = (uint32_t)wt << 18;
+                if (!q16) {
+                    const float f = (float)wt;
+                    std::memcpy(&bits, &f, 4);
+                }
+                r[0] = si * E;
+                r[1] = sj * E | bits;
+            }
+            if (lane == 31 || k + 1 == ec) at[(size_t)w] += 32 * RW;
+        }
+    }
+    for (int w = 0; w < W; ++w)
+        std::copy_n(rec.begin() + starts[(size_t)w],
+                    std::min(kRowsAhead * 32 * RW, at[(size_t)w] - starts[(size_t)w]), rec.begin() + at[(size_t)w]);
+    std::unique_ptr<RecordTable> t(new RecordTable());
+    t->K = h->K;
+    t->threads = h->threads;
+    t->format = h->format;
+    t->n_colours = nc;
+    int rc;
+    if ((rc = t->rec.ensure(rec.size())) || (rc = t->counts.ensure(counts.size())) ||
+        (rc = t->starts.ensure((size_t)W))) {
+        t->release();
+        return rc;
+    }
+    if (cudaMemcpy(t->rec.p, rec.data(), rec.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(t->counts.p, counts.data(), counts.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(t->starts.p, starts.data(), (size_t)W * 4, cudaMemcpyHostToDevice) != cudaSuccess) {
+        t->release();
+        return fail(COSM_ERR_CUDA, "copying the record table to the device failed");
+    }
+    h->table = t.get();
+    h->tables.push_back(std::move(t));
+    return COSM_OK;
+}
+
+int cosm::ensure_tables(cosm_handle *h)
+{
+    try {
+        if (h->shape >= 0) return ensure_patch_weights(h);
+        if (h->format >= 0) return ensure_records(h);
+    } catch (const std::bad_alloc &) {
+        return fail(COSM_ERR_NOMEM, "host allocation failed");
+    }
+    return COSM_OK;
+}
+
 // Replicas per CTA (K) and threads per CTA: maximise resident replicas per
 // SM (COSM_K / COSM_THREADS override for experiments).
 int cosm::choose_layout(cosm_handle *h, int replicas, bool narrow_ties)
@@ -678,8 +955,17 @@ int cosm::choose_layout(cosm_handle *h, int replicas, bool narrow_ties)
         h->staged = false;
         const size_t esz = p.storage == COSM_F32 ? 4 : 2;
         h->tile_stride = (int64_t)(((size_t)h->g.n * h->K * esz + 15) / 16 * 16 / esz);
-        return ensure_patch_weights(h);
+        h->format = -1;
+        return COSM_OK;
     }
+    if (mode == MODE_GENERAL_ && choose_edges(h, replicas, forceK, forceT)) {
+        h->block_pairs = false;
+        h->staged = false;
+        const size_t esz = p.storage == COSM_F32 ? 4 : 2;
+        h->tile_stride = (int64_t)(((size_t)h->g.n * h->K * esz + 15) / 16 * 16 / esz);
+        return COSM_OK;
+    }
+    h->format = -1;
     const bool pairs_ok = mode == MODE_LATTICE2D_ && p.storage == COSM_F32 && h->Wd % 2 == 0 &&
                           !std::getenv("COSM_SCALAR_F32") && !std::getenv("COSM_SINGLE_BLOCKS");
     long bestScore = -1;
@@ -839,6 +1125,12 @@ InstView cosm::inst_view(cosm_handle *h)
     v.wnib = h->d_wnib.p;
     v.Q = h->Q;
     v.Wd = h->Wd;
+    if (h->format >= 0 && h->table) {
+        v.rec = h->table->rec.p;
+        v.counts = h->table->counts.p;
+        v.starts = h->table->starts.p;
+        v.n_colours = h->table->n_colours;
+    }
     if (h->shape >= 0) {
         v.pwt = h->d_pwt[h->shape].p;
         v.pgr = h->pgr;
@@ -1066,7 +1358,7 @@ static int run_range(cosm_handle *h, int64_t sweeps, int64_t s0, int64_t s1, int
             return fail(COSM_ERR_INVALID_ARG, "a continued trial keeps its replica count and seed");
         if (h->stream && h->stream != st) CK(cudaStreamSynchronize(h->stream));
     } else if (!h->K || replicas != h->replicas) {
-        if ((rc = choose_layout(h, replicas))) return rc;
+        if ((rc = choose_layout(h, replicas)) || (rc = ensure_tables(h))) return rc;
     }
     h->replicas = replicas;
     h->seed = seed;
@@ -1109,7 +1401,7 @@ static int run_range(cosm_handle *h, int64_t sweeps, int64_t s0, int64_t s1, int
     a.segs = h->d_segs.p;
     a.seg_off = h->d_segoff.p;
     LaunchCfg cfg{h->mode, h->prm.storage, h->K, h->threads, (int)(h->h_segoff.size() - 1), h->smem, waits,
-                  h->shape, h->ragged};
+                  h->shape, h->ragged, h->format};
     h->grid = cfg.grid;
     if (kernel_launch(cfg, a, st))
         return fail(COSM_ERR_CUDA, std::string("sweep launch: ") + cudaGetErrorString(cudaGetLastError()));
@@ -1300,7 +1592,7 @@ extern "C" int cosm_set_state(cosm_handle *h, const double *phases, int32_t repl
     int rc;
     if (h->stream) CK(cudaStreamSynchronize(h->stream));
     if (!h->K || replicas != h->replicas) {
-        if ((rc = choose_layout(h, replicas))) return rc;
+        if ((rc = choose_layout(h, replicas)) || (rc = ensure_tables(h))) return rc;
     }
     h->replicas = replicas;
     h->seed = seed;
@@ -1379,7 +1671,7 @@ extern "C" int cosm_import_state(cosm_handle *h, const void *phases, int32_t sto
     int rc;
     if (h->stream) CK(cudaStreamSynchronize(h->stream));
     if (!h->K || replicas != h->replicas) {
-        if ((rc = choose_layout(h, replicas))) return rc;
+        if ((rc = choose_layout(h, replicas)) || (rc = ensure_tables(h))) return rc;
     }
     h->replicas = replicas;
     h->seed = seed;
@@ -1428,7 +1720,7 @@ static int launch_on_state(cosm_handle *h, int32_t flags, int64_t s0, int64_t s1
     a.v.S = s1;
     a.segs = h->d_segs.p;
     a.seg_off = h->d_segoff.p;
-    LaunchCfg cfg{h->mode, h->prm.storage, h->K, h->threads, (int)tiles, h->smem, false, h->shape, h->ragged};
+    LaunchCfg cfg{h->mode, h->prm.storage, h->K, h->threads, (int)tiles, h->smem, false, h->shape, h->ragged, h->format};
     h->grid = cfg.grid;
     if (kernel_launch(cfg, a, st))
         return fail(COSM_ERR_CUDA, std::string("sweep launch: ") + cudaGetErrorString(cudaGetLastError()));
@@ -1528,6 +1820,7 @@ struct BatchClass {
     int storage, K, mode;
     int shape;          // patch shape of lattices kept in registers (-1: none)
     bool ragged;
+    int format;         // record-table format of edge lists (-1: none)
     int threads;        // threads per CTA
     size_t smem;        // largest tile of the class
     int grid;           // CTAs (resident capacity, capped by units)
@@ -1654,15 +1947,64 @@ static int batch_instance_layout(cosm_batch *b, cosm_handle *h, int32_t replicas
         const int Kmin = h->prm.storage == COSM_F32 ? 1 : 2;
         const size_t esz = h->prm.storage == COSM_F32 ? 4 : 2;
         h->K = Kmin;
+        h->format = record_format(h, Kmin);
         h->block_pairs = false;
         h->staged = false;
         h->smem = sweep_smem_bytes(h->prm.storage, Kmin, h->g.n, h->prm.n_bisectors, h->mode);
         h->tile_stride = (int64_t)(((size_t)h->g.n * Kmin * esz + 15) / 16 * 16 / esz);
         // the narrow tile's kernel may allow fewer threads per CTA
-        while (h->threads > 64 && batch_occupancy(h->prm.storage, Kmin, h->mode, h->threads, h->smem) == 0)
-            h->threads /= 2;
-        h->occupancy = batch_occupancy(h->prm.storage, Kmin, h->mode, h->threads, h->smem);
+        while (h->threads > 64 && kernel_occupancy(h, h->threads, h->smem, true) == 0)
+            h->threads = half_threads(h->threads, h->format >= 0);
+        h->occupancy = kernel_occupancy(h, h->threads, h->smem, true);
     }
+    return COSM_OK;
+}
+
+// Runs work(t) for t = 0 .. workers - 1 on host threads, each with the
+// caller's device current.
+template <typename Work>
+static void on_workers(int workers, int dev, const Work &work)
+{
+    std::vector<std::thread> pool;
+    for (int t = 1; t < workers; ++t)
+        pool.emplace_back([&work, dev, t] {
+            cudaSetDevice(dev);
+            work(t);
+        });
+    work(0);
+    for (auto &th : pool) th.join();
+}
+
+// The device tables of every instance's layout. Missing ones (a first run, or
+// another layout) are built by host threads side by side.
+static int batch_tables(cosm_batch *b)
+{
+    std::vector<cosm_handle *> todo;
+    for (cosm_handle *h : b->hs) {
+        bool there = h->shape < 0 && h->format < 0;
+        if (h->shape >= 0) there = h->d_pwt[h->shape].p != nullptr;
+        for (size_t k = 0; k < h->tables.size() && h->format >= 0 && !there; ++k) {
+            const RecordTable &t = *h->tables[k];
+            there = t.K == h->K && t.threads == h->threads && t.format == h->format;
+        }
+        if (there) {
+            if (int rc = ensure_tables(h)) return rc;
+        } else {
+            todo.push_back(h);
+        }
+    }
+    if (todo.empty()) return COSM_OK;
+    int dev = 0;
+    CK(cudaGetDevice(&dev));
+    const int workers = (int)std::min<size_t>(todo.size(), std::max(1u, std::min(16u, std::thread::hardware_concurrency())));
+    std::vector<int> rcs(todo.size(), COSM_OK);
+    std::vector<std::string> msgs(todo.size());
+    on_workers(workers, dev, [&](int t) {
+        for (size_t i = (size_t)t; i < todo.size(); i += (size_t)workers)
+            if ((rcs[i] = ensure_tables(todo[i]))) msgs[i] = g_err;
+    });
+    for (size_t i = 0; i < todo.size(); ++i)
+        if (rcs[i]) return fail(rcs[i], msgs[i]);
     return COSM_OK;
 }
 
@@ -1680,13 +2022,17 @@ static int batch_layout(cosm_batch *b, const int64_t *sweeps, const int32_t *rep
         if ((rc = batch_instance_layout(b, h, replicas[i]))) return rc;
         if (b->threads && h->shape < 0) {
             h->threads = b->threads;
-            while (h->threads > 64 && batch_occupancy(h->prm.storage, h->K, h->mode, h->threads, h->smem) == 0)
-                h->threads /= 2;
+            while (h->threads > 64 && kernel_occupancy(h, h->threads, h->smem, true) == 0)
+                h->threads = half_threads(h->threads, h->format >= 0);
         }
         h->replicas = replicas[i];
         h->seed = seeds[i];
         if ((rc = ensure_run_buffers(h, replicas[i]))) return rc;
         if ((rc = upload_alpha(h, sweeps[i], st))) return rc;
+    }
+    if (int rc = batch_tables(b)) return rc;
+    for (int i = 0; i < n; ++i) {
+        cosm_handle *h = b->hs[(size_t)i];
         InstView v = inst_view(h);
         v.alpha_tab = h->d_alpha.p;
         v.alpha_base = 1;
@@ -1700,18 +2046,18 @@ static int batch_layout(cosm_batch *b, const int64_t *sweeps, const int32_t *rep
     // shared memory); their units form one queue, longest trials first
     b->classes.clear();
     b->h_units.clear();
-    struct Key { int storage, K, mode, shape; bool ragged; int threads, occ; };
+    struct Key { int storage, K, mode, shape; bool ragged; int format, threads, occ; };
     std::vector<Key> keys;
     std::vector<int> cls((size_t)n);
     for (int i = 0; i < n; ++i) {
         const cosm_handle *h = b->hs[(size_t)i];
-        const Key k{h->prm.storage, h->K, h->mode, h->shape, h->shape >= 0 && h->ragged, h->threads,
+        const Key k{h->prm.storage, h->K, h->mode, h->shape, h->shape >= 0 && h->ragged, h->format, h->threads,
                     kernel_occupancy(h, h->threads, h->smem, true)};
         int c = -1;
         for (size_t q = 0; q < keys.size() && c < 0; ++q) {
             const Key &o = keys[q];
             if (o.storage == k.storage && o.K == k.K && o.mode == k.mode && o.shape == k.shape && o.ragged == k.ragged &&
-                o.threads == k.threads && o.occ == k.occ)
+                o.format == k.format && o.threads == k.threads && o.occ == k.occ)
                 c = (int)q;
         }
         if (c < 0) {
@@ -1722,7 +2068,8 @@ static int batch_layout(cosm_batch *b, const int64_t *sweeps, const int32_t *rep
     }
     int dev_sms = b->hs[0]->num_sms;
     for (size_t c = 0; c < keys.size(); ++c) {
-        BatchClass bc{keys[c].storage, keys[c].K, keys[c].mode, keys[c].shape, keys[c].ragged, keys[c].threads, 0, 0,
+        BatchClass bc{keys[c].storage, keys[c].K, keys[c].mode, keys[c].shape, keys[c].ragged, keys[c].format,
+                      keys[c].threads, 0, 0,
                       (int32_t)b->h_units.size(), 0};
         std::vector<std::pair<double, BatchUnit>> us;
         for (int i = 0; i < n; ++i) {
@@ -1739,11 +2086,12 @@ static int batch_layout(cosm_batch *b, const int64_t *sweeps, const int32_t *rep
         bc.units = (int32_t)us.size();
         int T = bc.threads;
         const auto occ_of = [&](int threads) {
-            return bc.shape >= 0 ? patch_occupancy(bc.storage, bc.K, bc.shape, bc.ragged, threads, bc.smem)
-                                 : batch_occupancy(bc.storage, bc.K, bc.mode, threads, bc.smem);
+            return bc.shape >= 0    ? patch_occupancy(bc.storage, bc.K, bc.shape, bc.ragged, threads, bc.smem)
+                   : bc.format >= 0 ? edges_occupancy(bc.storage, bc.K, bc.format, threads, bc.smem)
+                                    : batch_occupancy(bc.storage, bc.K, bc.mode, threads, bc.smem);
         };
         int occ = occ_of(T);
-        while (occ == 0 && T > 64 && bc.shape < 0) {
+        while (occ == 0 && T > 64 && bc.shape < 0 && bc.format < 0) {  // tables are laid out for T
             T /= 2;
             occ = occ_of(T);
         }
@@ -1785,7 +2133,7 @@ static int batch_enqueue(cosm_batch *b, cudaStream_t st)
         CK(cudaStreamWaitEvent(b->side[c], b->ev[0], 0));
         BatchArgs a{b->d_insts.p, b->d_units.p + bc.unit0, bc.units, b->d_counters.p + c};
         if (bc.units > 0 && kernel_launch_queue(LaunchCfg{bc.mode, bc.storage, bc.K, bc.threads, bc.grid, bc.smem, false, bc.shape,
-                                                       bc.ragged}, a, b->side[c]))
+                                                       bc.ragged, bc.format}, a, b->side[c]))
             return fail(COSM_ERR_CUDA, std::string("batch launch: ") + cudaGetErrorString(cudaGetLastError()));
         CK(cudaEventRecord(b->ev[c + 1], b->side[c]));
     }
@@ -1816,7 +2164,7 @@ extern "C" int cosm_batch_run(cosm_batch *b, const int64_t *sweeps, const int32_
     sig.push_back((int64_t)(uintptr_t)b->d_counters.p);
     for (const BatchClass &bc : b->classes) {
         sig.push_back(bc.storage); sig.push_back(bc.K); sig.push_back(bc.mode); sig.push_back(bc.threads);
-        sig.push_back(bc.shape); sig.push_back(bc.ragged);
+        sig.push_back(bc.shape); sig.push_back(bc.ragged); sig.push_back(bc.format);
         sig.push_back((int64_t)bc.smem); sig.push_back(bc.grid); sig.push_back(bc.unit0); sig.push_back(bc.units);
     }
     if (!b->exec || sig != b->sig) {

@@ -119,7 +119,7 @@ static int admit(cosm_server *s, Request *r)
     for (int k = 0; k < 3; ++k) d.dims[k] = r->dims[k];
     int rc = cosm_create(&d, &r->prm, &r->h);
     if (rc) return rc;
-    if ((rc = choose_layout(r->h, r->R))) return rc;
+    if ((rc = choose_layout(r->h, r->R)) || (rc = ensure_tables(r->h))) return rc;
     r->h->replicas = r->R;
     if ((rc = ensure_run_buffers(r->h, r->R))) return rc;
     if ((rc = upload_alpha(r->h, r->S, s->st))) return rc;
@@ -145,7 +145,9 @@ static int run_chunk(cosm_server *s, const std::vector<Request *> &act)
 {
     const int n = (int)act.size();
     std::vector<InstView> views((size_t)n);
-    struct Key { int storage, K, mode, shape; bool ragged; int threads; };  // threads: of the patch shape
+    // classes: one kernel and thread count each (patch shapes and record tables
+    // have their own; the others a count for the class)
+    struct Key { int storage, K, mode, shape; bool ragged; int format, threads; };
     std::vector<Key> keys;
     std::vector<std::vector<BatchUnit>> per;
     std::vector<size_t> smem;
@@ -155,17 +157,25 @@ static int run_chunk(cosm_server *s, const std::vector<Request *> &act)
         Request *r = act[(size_t)i];
         cosm_handle *h = r->h;
         h->seed = trial_seed(r->seed, r->trial);
+        int rc;
+        if (h->format >= 0 && s->cfg.threads) {
+            h->threads = (s->cfg.threads + 31) / 32 * 32;  // whole warps
+            while (h->threads > 64 && kernel_occupancy(h, h->threads, h->smem, true) == 0)
+                h->threads = half_threads(h->threads, true);
+        }
+        if ((rc = ensure_tables(h))) return rc;
         InstView v = inst_view(h);
         v.alpha_tab = h->d_alpha.p;
         v.alpha_base = 1;
         v.S = r->S;
         views[(size_t)i] = v;
         int c = -1;
-        const Key own{h->prm.storage, h->K, h->mode, h->shape, h->shape >= 0 && h->ragged,
-                      h->shape >= 0 ? h->threads : 0};
+        const Key own{h->prm.storage, h->K, h->mode, h->shape, h->shape >= 0 && h->ragged, h->format,
+                      h->shape >= 0 || h->format >= 0 ? h->threads : 0};
         for (size_t k = 0; k < keys.size(); ++k)
             if (keys[k].storage == own.storage && keys[k].K == own.K && keys[k].mode == own.mode &&
-                keys[k].shape == own.shape && keys[k].ragged == own.ragged && keys[k].threads == own.threads)
+                keys[k].shape == own.shape && keys[k].ragged == own.ragged && keys[k].format == own.format &&
+                keys[k].threads == own.threads)
                 c = (int)k;
         if (c < 0) {
             keys.push_back(own);
@@ -207,7 +217,6 @@ static int run_chunk(cosm_server *s, const std::vector<Request *> &act)
     }
     if (keys.size() > 1) CK(cudaEventRecord(s->ev[0], s->st));
     for (size_t c = 0; c < keys.size(); ++c) {
-        // a patch shape has its own thread count
         int T = keys[c].threads ? keys[c].threads
                 : s->cfg.threads ? s->cfg.threads
                                  : std::min(512, std::max(64, ((max_ec[c] + 1) / 2 + 31) / 32 * 32));
@@ -224,7 +233,7 @@ static int run_chunk(cosm_server *s, const std::vector<Request *> &act)
         cudaStream_t st = c ? s->side[c - 1] : s->st;
         if (c > 0) CK(cudaStreamWaitEvent(st, s->ev[0], 0));
         if (kernel_launch_queue(LaunchCfg{keys[c].mode, keys[c].storage, keys[c].K, T, grid, smem[c], false,
-                                          keys[c].shape, keys[c].ragged}, a, st))
+                                          keys[c].shape, keys[c].ragged, keys[c].format}, a, st))
             return fail(COSM_ERR_CUDA, std::string("serving launch: ") + cudaGetErrorString(cudaGetLastError()));
         s->launches++;
         if (c > 0) CK(cudaEventRecord(s->ev[c], st));
