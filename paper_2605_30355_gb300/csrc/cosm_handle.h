@@ -136,6 +136,7 @@ struct cosm_handle {
     DevBuf<uint32_t> d_qbuf;        // optimal bisector scratch
     DevBuf<int32_t> d_delta;
     DevBuf<uint64_t> d_items;
+    DevBuf<unsigned char> d_stage;  // rows on their way in or out (bounded, state_rows)
     int32_t n_trace = 0;            // readouts per trial of the last tracked run
     bool have_trace = false;
     bool bits_valid = false;        // d_bits holds the kept spins of the last run

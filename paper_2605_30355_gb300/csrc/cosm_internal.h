@@ -208,6 +208,20 @@ struct FinalArgs {
 };
 int finalize_launch(const FinalArgs &a, void *stream);
 
+// State between the tile layout [tile][slot][K] and rows [replica][vertex] in
+// original vertex order, for the tiles t0 .. t0 + tiles - 1 (rows holds their
+// first replica's row first).
+enum StateKind { STATE_RAW = 0, STATE_TURNS = 1 };  // storage type, or binary64 turns in [0, 1)
+struct StateArgs {
+    void *state;
+    int64_t stride;          // storage elements per tile
+    const int32_t *orig_of;
+    void *rows;
+    int32_t storage, K, n, replicas, t0, tiles;
+};
+int state_export_launch(const StateArgs &a, int kind, void *stream);
+int state_import_launch(const StateArgs &a, void *stream);
+
 // Optimal-bisector readout (Section II-B; Burer, Monteiro and Zhang 2002):
 // per replica, the best cut over every bisector position, from the stored
 // phases; one CTA per replica at a time, scratch in global memory.

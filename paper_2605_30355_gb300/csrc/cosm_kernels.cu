@@ -1,6 +1,8 @@
 // CUDA kernels of Cosm for sm_103a: the sweep kernels of edge lists and of
 // lattices kept in shared memory, the finalisers, the optimal-bisector
 // readout and the measurement probes.
+#include <algorithm>
+
 #include "cosm_device.cuh"
 
 namespace cosm {
@@ -225,6 +227,112 @@ __global__ void __launch_bounds__(1024) opt_readout_kernel(const OptArgs o)
         }
         __syncthreads();
     }
+}
+
+// ---------------------------------------------------------------- state in and out
+// A thread takes one slot of one tile: one vector access to its K phases in
+// the tile layout, K scalar ones to the replicas' rows (neighbouring slots'
+// vertices lie one or two apart). Bound by HBM: a few tens of microseconds
+// for 256 replicas of 20,000 phases, where the host loop over the copied
+// state took 12 ms.
+template <typename T, int K>
+struct __align__(sizeof(T) * K) Lanes {
+    T v[K];
+};
+
+__device__ __forceinline__ double turn_of(double g)
+{
+    const double x = g - floor(g);
+    return x >= 1.0 ? 0.0 : x;
+}
+template <int kStorage, typename T>
+__device__ __forceinline__ double stored_turn(T raw)
+{
+    if constexpr (kStorage == 0) return turn_of((double)__uint_as_float(raw));
+    else if constexpr (kStorage == 1) return turn_of((double)__half2float(__ushort_as_half(raw)));
+    else if constexpr (kStorage == 3) return turn_of((double)__bfloat162float(__ushort_as_bfloat16(raw)));
+    else return (double)raw / 65536.0;  // fixed point: already a turn in [0, 1)
+}
+
+// kStorage -1: the storage type itself.
+template <typename T, int K, int kStorage>
+__global__ void __launch_bounds__(256) state_export_kernel(const StateArgs a)
+{
+    const int slot = blockIdx.x * blockDim.x + threadIdx.x;
+    if (slot >= a.n) return;
+    const int v = a.orig_of[slot];
+    for (int t = blockIdx.y; t < a.tiles; t += gridDim.y) {
+        const Lanes<T, K> x = reinterpret_cast<const Lanes<T, K> *>(
+            reinterpret_cast<const T *>(a.state) + (size_t)(a.t0 + t) * (size_t)a.stride)[slot];
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int64_t r = (int64_t)t * K + k;  // row
+            if ((int64_t)a.t0 * K + r >= a.replicas) break;
+            if constexpr (kStorage < 0) reinterpret_cast<T *>(a.rows)[r * a.n + v] = x.v[k];
+            else reinterpret_cast<double *>(a.rows)[r * a.n + v] = stored_turn<kStorage>(x.v[k]);
+        }
+    }
+}
+
+// Replicas past the last one, and places past the last slot, become zero.
+template <typename T, int K>
+__global__ void __launch_bounds__(256) state_import_kernel(const StateArgs a)
+{
+    const int slot = blockIdx.x * blockDim.x + threadIdx.x;
+    if ((int64_t)slot * K >= a.stride) return;
+    const int v = slot < a.n ? a.orig_of[slot] : 0;
+    for (int t = blockIdx.y; t < a.tiles; t += gridDim.y) {
+        T *tile = reinterpret_cast<T *>(a.state) + (size_t)(a.t0 + t) * (size_t)a.stride;
+        Lanes<T, K> x;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int64_t r = (int64_t)t * K + k;
+            const bool there = slot < a.n && (int64_t)a.t0 * K + r < a.replicas;
+            x.v[k] = there ? reinterpret_cast<const T *>(a.rows)[r * a.n + v] : (T)0;
+        }
+        if ((int64_t)(slot + 1) * K <= a.stride) {
+            reinterpret_cast<Lanes<T, K> *>(tile)[slot] = x;
+        } else {
+            for (int64_t k = 0; (int64_t)slot * K + k < a.stride; ++k) tile[(int64_t)slot * K + k] = x.v[k];
+        }
+    }
+}
+
+template <typename T, int K>
+static int state_launch(const StateArgs &a, int what, cudaStream_t st)
+{
+    const int64_t slots = what < 0 ? (a.stride + K - 1) / K : a.n;
+    const dim3 grid((unsigned)((slots + 255) / 256), (unsigned)std::min(a.tiles, 4096));
+    if (what < 0) state_import_kernel<T, K><<<grid, 256, 0, st>>>(a);
+    else if (what == STATE_RAW) state_export_kernel<T, K, -1><<<grid, 256, 0, st>>>(a);
+    else if constexpr (sizeof(T) == 4) state_export_kernel<T, K, 0><<<grid, 256, 0, st>>>(a);
+    else if (a.storage == 1) state_export_kernel<T, K, 1><<<grid, 256, 0, st>>>(a);
+    else if (a.storage == 3) state_export_kernel<T, K, 3><<<grid, 256, 0, st>>>(a);
+    else state_export_kernel<T, K, 2><<<grid, 256, 0, st>>>(a);
+    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+static int state_dispatch(const StateArgs &a, int what, cudaStream_t st)
+{
+    if (a.storage == 0) {
+        if (a.K == 1) return state_launch<uint32_t, 1>(a, what, st);
+        if (a.K == 2) return state_launch<uint32_t, 2>(a, what, st);
+        if (a.K == 4) return state_launch<uint32_t, 4>(a, what, st);
+    } else {
+        if (a.K == 2) return state_launch<uint16_t, 2>(a, what, st);
+        if (a.K == 4) return state_launch<uint16_t, 4>(a, what, st);
+        if (a.K == 8) return state_launch<uint16_t, 8>(a, what, st);
+    }
+    return -1;
+}
+
+int state_export_launch(const StateArgs &a, int kind, void *stream)
+{
+    return state_dispatch(a, kind, reinterpret_cast<cudaStream_t>(stream));
+}
+int state_import_launch(const StateArgs &a, void *stream)
+{
+    return state_dispatch(a, -1, reinterpret_cast<cudaStream_t>(stream));
 }
 
 // ---------------------------------------------------------------- host side

@@ -142,7 +142,7 @@ extern "C" void cosm_destroy(cosm_handle *h)
     for (auto &b : h->d_pwt) b.release();
     for (auto &t : h->tables) t->release();
     h->d_h.release(); h->d_energy.release(); h->d_bisB.release(); h->d_trace.release();
-    h->d_bits.release(); h->d_qbuf.release(); h->d_delta.release(); h->d_items.release();
+    h->d_bits.release(); h->d_qbuf.release(); h->d_delta.release(); h->d_items.release(); h->d_stage.release();
     delete h;
 }
 
@@ -1536,13 +1536,30 @@ extern "C" int cosm_get_replica_cuts(cosm_handle *h, int64_t *cuts, int32_t *bes
     return COSM_OK;
 }
 
-// Stored value (FP32 or FP16, representative in [-1/2, 1/2]) -> turn in [0, 1).
-// Turn in [0, 1) of a stored representative (binary32 lattice phases may sit
-// anywhere in (-1, 1) between wraps).
-static inline double to_turn(double g)
+// Moves the state between the device's tile layout and rows [replica][vertex]
+// of the caller (host or device), a few tiles at a time through a staging
+// buffer of at most 64 MB: kind >= 0 exports (StateKind), -1 imports.
+static int state_rows(cosm_handle *h, int kind, void *rows)
 {
-    const double x = g - std::floor(g);
-    return x >= 1.0 ? 0.0 : x;
+    const size_t esz = kind == STATE_TURNS ? 8 : (h->prm.storage == COSM_F32 ? 4 : 2);
+    const size_t row = (size_t)h->g.n * esz;
+    const int64_t tiles = (h->replicas + h->K - 1) / h->K;
+    int64_t step = std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)(((size_t)64 << 20) / (row * h->K))));
+    int rc;
+    while ((rc = h->d_stage.ensure((size_t)step * h->K * row)) && step > 1) step = (step + 1) / 2;
+    if (rc) return rc;
+    for (int64_t t0 = 0; t0 < tiles; t0 += step) {
+        const int64_t r0 = t0 * h->K, r1 = std::min<int64_t>(h->replicas, (t0 + step) * h->K);
+        unsigned char *part = static_cast<unsigned char *>(rows) + (size_t)r0 * row;
+        StateArgs a{h->d_state.p, h->tile_stride, h->d_orig.p, h->d_stage.p, h->prm.storage, h->K, h->g.n,
+                    h->replicas, (int32_t)t0, (int32_t)std::min<int64_t>(step, tiles - t0)};
+        if (kind < 0) CK(cudaMemcpy(h->d_stage.p, part, (size_t)(r1 - r0) * row, cudaMemcpyDefault));
+        if (kind < 0 ? state_import_launch(a, nullptr) : state_export_launch(a, kind, nullptr))
+            return fail(COSM_ERR_CUDA, std::string("state launch: ") + cudaGetErrorString(cudaGetLastError()));
+        if (kind >= 0) CK(cudaMemcpy(part, h->d_stage.p, (size_t)(r1 - r0) * row, cudaMemcpyDefault));
+    }
+    CK(cudaStreamSynchronize(nullptr));
+    return COSM_OK;
 }
 
 extern "C" int cosm_get_state(cosm_handle *h, double *phases)
@@ -1551,38 +1568,7 @@ extern "C" int cosm_get_state(cosm_handle *h, double *phases)
     if (!h->have_state) return fail(COSM_ERR_STATE, "no state yet");
     int rc = cosm_sync(h);
     if (rc) return rc;
-    const int64_t tiles = (h->replicas + h->K - 1) / h->K;
-    const size_t esz = h->prm.storage == COSM_F32 ? 4 : 2;
-    std::vector<unsigned char> raw((size_t)tiles * (size_t)h->tile_stride * esz);
-    CK(cudaMemcpy(raw.data(), h->d_state.p, raw.size(), cudaMemcpyDeviceToHost));
-    std::vector<double> out((size_t)h->replicas * h->g.n);
-    for (int32_t r = 0; r < h->replicas; ++r) {
-        const size_t base = (size_t)(r / h->K) * (size_t)h->tile_stride;
-        for (int32_t v = 0; v < h->g.n; ++v) {
-            const size_t idx = base + (size_t)h->slot_of[(size_t)v] * h->K + (size_t)(r % h->K);
-            double g;
-            if (esz == 4) {
-                float f;
-                std::memcpy(&f, raw.data() + idx * 4, 4);
-                g = f;
-            } else if (h->prm.storage == COSM_BF16) {
-                __nv_bfloat16 bv;
-                std::memcpy(&bv, raw.data() + idx * 2, 2);
-                g = (double)__bfloat162float(bv);
-            } else if (h->prm.storage == COSM_F16) {
-                __half hv;
-                std::memcpy(&hv, raw.data() + idx * 2, 2);
-                g = (double)__half2float(hv);
-            } else {
-                uint16_t q;
-                std::memcpy(&q, raw.data() + idx * 2, 2);
-                g = (double)q / 65536.0;  // fixed point: already a turn in [0, 1)
-            }
-            out[(size_t)r * h->g.n + v] = to_turn(g);
-        }
-    }
-    CK(cudaMemcpy(phases, out.data(), out.size() * 8, cudaMemcpyDefault));
-    return COSM_OK;
+    return state_rows(h, STATE_TURNS, phases);
 }
 
 extern "C" int cosm_set_state(cosm_handle *h, const double *phases, int32_t replicas, uint64_t seed)
@@ -1633,10 +1619,6 @@ extern "C" int cosm_set_state(cosm_handle *h, const double *phases, int32_t repl
     return COSM_OK;
 }
 
-// Checkpoint of the state in its storage type: element (r, v) of the tile
-// layout [tile][slot][K] <-> [replica][vertex] in original vertex order.
-static size_t storage_bytes(int storage) { return storage == COSM_F32 ? 4 : 2; }
-
 extern "C" int cosm_export_state(cosm_handle *h, void *phases, int32_t storage, int64_t *sweep_idx)
 {
     if (!h || !phases) return fail(COSM_ERR_INVALID_ARG, "NULL argument");
@@ -1644,19 +1626,7 @@ extern "C" int cosm_export_state(cosm_handle *h, void *phases, int32_t storage, 
     if (!h->have_state) return fail(COSM_ERR_STATE, "no state yet");
     int rc = cosm_sync(h);
     if (rc) return rc;
-    const int64_t tiles = (h->replicas + h->K - 1) / h->K;
-    const size_t esz = storage_bytes(storage);
-    std::vector<unsigned char> raw((size_t)tiles * (size_t)h->tile_stride * esz);
-    CK(cudaMemcpy(raw.data(), h->d_state.p, raw.size(), cudaMemcpyDeviceToHost));
-    std::vector<unsigned char> out((size_t)h->replicas * h->g.n * esz);
-    for (int32_t r = 0; r < h->replicas; ++r) {
-        const size_t base = (size_t)(r / h->K) * (size_t)h->tile_stride;
-        for (int32_t v = 0; v < h->g.n; ++v) {
-            const size_t idx = base + (size_t)h->slot_of[(size_t)v] * h->K + (size_t)(r % h->K);
-            std::memcpy(out.data() + ((size_t)r * h->g.n + v) * esz, raw.data() + idx * esz, esz);
-        }
-    }
-    CK(cudaMemcpy(phases, out.data(), out.size(), cudaMemcpyDefault));
+    if ((rc = state_rows(h, STATE_RAW, phases))) return rc;
     if (sweep_idx) *sweep_idx = h->sweep_idx;
     return COSM_OK;
 }
@@ -1676,19 +1646,7 @@ extern "C" int cosm_import_state(cosm_handle *h, const void *phases, int32_t sto
     h->replicas = replicas;
     h->seed = seed;
     if ((rc = ensure_run_buffers(h, replicas))) return rc;
-    const size_t esz = storage_bytes(storage);
-    std::vector<unsigned char> in((size_t)replicas * h->g.n * esz);
-    CK(cudaMemcpy(in.data(), phases, in.size(), cudaMemcpyDefault));
-    const int64_t tiles = (replicas + h->K - 1) / h->K;
-    std::vector<unsigned char> raw((size_t)tiles * (size_t)h->tile_stride * esz, 0);
-    for (int32_t r = 0; r < replicas; ++r) {
-        const size_t base = (size_t)(r / h->K) * (size_t)h->tile_stride;
-        for (int32_t v = 0; v < h->g.n; ++v) {
-            const size_t idx = base + (size_t)h->slot_of[(size_t)v] * h->K + (size_t)(r % h->K);
-            std::memcpy(raw.data() + idx * esz, in.data() + ((size_t)r * h->g.n + v) * esz, esz);
-        }
-    }
-    CK(cudaMemcpy(h->d_state.p, raw.data(), raw.size(), cudaMemcpyHostToDevice));
+    if ((rc = state_rows(h, -1, const_cast<void *>(phases)))) return rc;
     h->have_state = true;
     h->sweep_idx = sweep_idx;
     h->have_result = false;
