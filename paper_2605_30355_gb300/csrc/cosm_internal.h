@@ -229,8 +229,7 @@ struct OptArgs {
     InstView v;           // graph, state, outputs
     uint32_t *qbuf;       // [grid][n] phase positions of the current replica
     int32_t *delta;       // [grid][n] cut change at each vertex's position
-    uint64_t *items;      // [grid][npow2] (position << 32 | delta), sorted
-    int32_t npow2;        // power of two >= n
+    uint64_t *items;      // [grid][2][n] (position << 32 | delta), the sort's two buffers
     int32_t keep_better;  // 1: replace the kept readout only if strictly lower in energy
     int32_t storage;      // 0 f32, 1 f16, 2 u16 fixed point
     int32_t pad_;

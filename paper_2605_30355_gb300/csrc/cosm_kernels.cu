@@ -95,30 +95,123 @@ __global__ void __launch_bounds__(1024) batch_finalize_kernel(const InstView *in
 // bit of q_v, s_v(B) = +1 iff [B <= phi_v] xor t_v for B in [0, 2^31), so an
 // edge's cut state flips on the interval (lo, hi] of its endpoints'
 // positions: d_e = w_e (1 - 2 (t_i xor t_j)) enters at lo + 1 and leaves at
-// hi + 1. Each vertex collects the changes that happen at its position,
-// the (position, change) pairs are sorted (bitonic network over a power of
-// two, in global scratch), and a block-wide prefix sum gives the cut at
-// every position where it can change; the best (ties: the smallest B)
-// competes with the replica's kept readout.
-__global__ void __launch_bounds__(1024) opt_readout_kernel(const OptArgs o)
+// hi + 1. Each vertex collects the changes that happen at its position, the
+// (position, change) pairs are sorted by position, and a block-wide prefix sum
+// gives the cut at every position where it can change; the best (ties: the
+// smallest B) competes with the replica's kept readout.
+//
+// One CTA of 1,024 threads per replica at a time, one CTA per SM. The changes
+// are summed with shared-memory atomics (global ones where 8 n bytes do not
+// fit) and sorted by a least-significant-digit radix sort, 8 bits a pass: each
+// warp ranks a contiguous chunk against per-warp digit counts in shared
+// memory (match.any orders equal digits), and scatters it to one of two
+// buffers in global memory, which stay in L2. Digits in which no two positions
+// differ are skipped (fixed point: the lower 16 bits). A bitonic network over
+// global memory with a serial block scan took 1.18 ms per replica of 20,000
+// vertices and 40,000 edges.
+constexpr int kOptThreads = 1024, kOptWarps = kOptThreads / 32, kDigits = 256;
+
+__device__ __forceinline__ long long block_exclusive_sum(long long x, long long *warp_sums)
 {
-    __shared__ long long s_part[1024];
-    __shared__ long long s_best[1024];
-    __shared__ uint32_t s_B[1024];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    long long inc = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    if (lane == 31) warp_sums[w] = inc;
+    __syncthreads();
+    if (w == 0) {
+        long long s = warp_sums[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long y = __shfl_up_sync(0xFFFFFFFFu, s, o);
+            if (lane >= o) s += y;
+        }
+        warp_sums[lane] = s;
+    }
+    __syncthreads();
+    const long long before = w ? warp_sums[w - 1] : 0;
+    __syncthreads();  // warp_sums may be used again
+    return before + inc - x;
+}
+
+// One pass of the sort on the digit at `shift`: elements get(i), i < n, into
+// out. hist: kDigits x 33 words of shared memory.
+template <typename Get>
+__device__ __forceinline__ void radix_pass(int n, int shift, uint32_t *hist, long long *warp_sums, uint64_t *out,
+                                           const Get &get)
+{
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    for (int i = tid; i < kDigits * 33; i += kOptThreads) hist[i] = 0u;
+    __syncthreads();
+    const int chunk = ((n + kOptWarps - 1) / kOptWarps + 31) / 32 * 32;
+    const int i0 = w * chunk, i1 = min(n, i0 + chunk);
+    for (int i = i0; i < i1; i += 32) {
+        const bool in = i + lane < i1;
+        const uint32_t d = in ? (uint32_t)(get(i + lane) >> (32 + shift)) & 0xFFu : 0xFFFFFFFFu;
+        const uint32_t same = __match_any_sync(0xFFFFFFFFu, d);
+        if (in && lane == __ffs(same) - 1) hist[d * 33 + w] += __popc(same);
+        __syncwarp();
+    }
+    __syncthreads();
+    // offsets in (digit, warp) order: eight counts per thread
+    {
+        uint32_t *h = hist + (tid >> 2) * 33 + (tid & 3) * 8;
+        uint32_t c[8], sum = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            c[k] = h[k];
+            sum += c[k];
+        }
+        uint32_t at = (uint32_t)block_exclusive_sum(sum, warp_sums);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            h[k] = at;
+            at += c[k];
+        }
+    }
+    __syncthreads();
+    for (int i = i0; i < i1; i += 32) {
+        const bool in = i + lane < i1;
+        const uint64_t x = in ? get(i + lane) : 0ull;
+        const uint32_t d = in ? (uint32_t)(x >> (32 + shift)) & 0xFFu : 0xFFFFFFFFu;
+        const uint32_t same = __match_any_sync(0xFFFFFFFFu, d);
+        if (in) out[hist[d * 33 + w] + __popc(same & ((1u << lane) - 1u))] = x;
+        __syncwarp();
+        if (in && lane == __ffs(same) - 1) hist[d * 33 + w] += __popc(same);
+        __syncwarp();
+    }
+    __syncthreads();
+}
+
+template <bool kShared>
+__global__ void __launch_bounds__(kOptThreads) opt_readout_kernel(const OptArgs o)
+{
+    extern __shared__ __align__(16) uint32_t opt_smem[];
+    __shared__ long long s_sums[kOptWarps], s_best[kOptWarps];
+    __shared__ uint32_t s_B[kOptWarps];
     __shared__ unsigned long long s_c0;
+    __shared__ uint32_t s_diff;
     __shared__ int s_take;
     const InstView &v = o.v;
-    const int tid = threadIdx.x, nt = blockDim.x, n = v.n, N = o.npow2;
-    uint32_t *qb = o.qbuf + (size_t)blockIdx.x * n;
-    int32_t *dl = o.delta + (size_t)blockIdx.x * n;
-    uint64_t *it = o.items + (size_t)blockIdx.x * N;
+    constexpr int nt = kOptThreads;
+    const int tid = threadIdx.x, lane = tid & 31, n = v.n;
+    uint32_t *hist = opt_smem;
+    uint32_t *qb = kShared ? opt_smem + kDigits * 33 : o.qbuf + (size_t)blockIdx.x * n;
+    int32_t *dl = kShared ? reinterpret_cast<int32_t *>(qb + n) : o.delta + (size_t)blockIdx.x * n;
+    uint64_t *const buf0 = o.items + (size_t)blockIdx.x * 2 * n, *const buf1 = buf0 + n;
     const int m = __ldg(v.off + v.C);
     const int storage = o.storage;
     for (int r = blockIdx.x; r < v.replicas; r += gridDim.x) {
-        const int tile = r / v.K, lane = r % v.K;
-        if (tid == 0) s_c0 = 0ull;
+        const int tile = r / v.K, place = r % v.K;
+        if (tid == 0) {
+            s_c0 = 0ull;
+            s_diff = 0u;
+        }
         for (int u = tid; u < n; u += nt) {
-            qb[u] = stored_q(v.state, storage, (size_t)tile * v.state_tile_stride + (size_t)u * v.K + lane);
+            qb[u] = stored_q(v.state, storage, (size_t)tile * v.state_tile_stride + (size_t)u * v.K + place);
             dl[u] = 0;
         }
         __syncthreads();
@@ -138,44 +231,37 @@ __global__ void __launch_bounds__(1024) opt_readout_kernel(const OptArgs o)
         }
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) c0 += __shfl_xor_sync(0xFFFFFFFFu, c0, off);
-        if ((tid & 31) == 0) atomicAdd(&s_c0, (unsigned long long)c0);
+        if (lane == 0) atomicAdd(&s_c0, (unsigned long long)c0);
+        uint32_t diff = 0;
+        const uint32_t first = qb[0];
+        for (int u = tid; u < n; u += nt) diff |= qb[u] ^ first;
+        diff = __reduce_or_sync(0xFFFFFFFFu, diff);
+        if (lane == 0) atomicOr(&s_diff, diff);
         __syncthreads();
-        for (int u = tid; u < N; u += nt)
-            it[u] = u < n ? ((uint64_t)(qb[u] & 0x7FFFFFFFu) << 32) | (uint32_t)dl[u] : 0xFFFFFFFF00000000ull;
-        __syncthreads();
-        for (int k = 2; k <= N; k <<= 1) {
-            for (int j = k >> 1; j > 0; j >>= 1) {
-                for (int i = tid; i < N; i += nt) {
-                    const int l = i ^ j;
-                    if (l > i) {
-                        const uint64_t x = it[i], y = it[l];
-                        if ((x > y) == ((i & k) == 0)) {
-                            it[i] = y;
-                            it[l] = x;
-                        }
-                    }
-                }
-                __syncthreads();
+        const uint32_t digits = s_diff;
+        // the sort: the first pass reads the vertices, the others a buffer
+        uint64_t *it = nullptr;
+#pragma unroll 1
+        for (int shift = 0; shift < 32; shift += 8) {
+            if (!((digits & 0x7FFFFFFFu) >> shift & 0xFFu) && !(shift == 24 && !it)) continue;
+            uint64_t *out = it == buf0 ? buf1 : buf0;
+            if (it) {
+                const uint64_t *in = it;
+                radix_pass(n, shift, hist, s_sums, out, [in](int i) { return in[i]; });
+            } else {
+                radix_pass(n, shift, hist, s_sums, out, [qb, dl](int i) {
+                    return ((uint64_t)(qb[i] & 0x7FFFFFFFu) << 32) | (uint32_t)dl[i];
+                });
             }
+            it = out;
         }
         // block prefix sum over contiguous chunks of the sorted pairs
         const int chunk = (n + nt - 1) / nt;
         const int a0 = min(n, tid * chunk), a1 = min(n, a0 + chunk);
         long long sum = 0;
         for (int i = a0; i < a1; ++i) sum += (int32_t)(uint32_t)it[i];
-        s_part[tid] = sum;
-        __syncthreads();
-        if (tid == 0) {
-            long long acc = 0;
-            for (int i = 0; i < nt; ++i) {
-                const long long t0 = s_part[i];
-                s_part[i] = acc;
-                acc += t0;
-            }
-        }
-        __syncthreads();
         const long long C0 = (long long)s_c0;
-        long long run = C0 + s_part[tid], best = LLONG_MIN;
+        long long run = C0 + block_exclusive_sum(sum, s_sums), best = LLONG_MIN;
         uint32_t bB = 0xFFFFFFFFu;
         if (tid == 0) { best = C0; bB = 0; }
         for (int i = a0; i < a1; ++i) {
@@ -188,35 +274,46 @@ __global__ void __launch_bounds__(1024) opt_readout_kernel(const OptArgs o)
                 bB = pos + 1u;
             }
         }
-        s_best[tid] = best;
-        s_B[tid] = bB;
-        __syncthreads();
-        for (int off = nt / 2; off > 0; off >>= 1) {
-            if (tid < off) {
-                const long long c = s_best[tid + off];
-                const uint32_t b2 = s_B[tid + off];
-                if (c > s_best[tid] || (c == s_best[tid] && b2 < s_B[tid])) {
-                    s_best[tid] = c;
-                    s_B[tid] = b2;
-                }
+        const auto better = [&](long long c, uint32_t b2) {
+            if (c > best || (c == best && b2 < bB)) {
+                best = c;
+                bB = b2;
             }
-            __syncthreads();
+        };
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            const long long c = __shfl_xor_sync(0xFFFFFFFFu, best, off);
+            better(c, __shfl_xor_sync(0xFFFFFFFFu, bB, off));
         }
-        const long long cut = s_best[0];
-        const uint32_t B = s_B[0];
-        if (tid == 0) {
-            const long long E = v.W - 2 * cut;
-            const int take = !o.keep_better || !v.energy || E < v.energy[r];
-            if (take) {
-                v.cut[r] = cut;
-                v.bestp[r] = -1;
-                if (v.energy) v.energy[r] = E;
-                if (v.bisB) v.bisB[r] = B;
+        if (lane == 0) {
+            s_best[tid >> 5] = best;
+            s_B[tid >> 5] = bB;
+        }
+        __syncthreads();
+        if (tid < 32) {
+            best = s_best[lane];
+            bB = s_B[lane];
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                const long long c = __shfl_xor_sync(0xFFFFFFFFu, best, off);
+                better(c, __shfl_xor_sync(0xFFFFFFFFu, bB, off));
             }
-            s_take = take;
+            if (tid == 0) {
+                s_B[0] = bB;
+                const long long E = v.W - 2 * best;
+                const int take = !o.keep_better || !v.energy || E < v.energy[r];
+                if (take) {
+                    v.cut[r] = best;
+                    v.bestp[r] = -1;
+                    if (v.energy) v.energy[r] = E;
+                    if (v.bisB) v.bisB[r] = bB;
+                }
+                s_take = take;
+            }
         }
         __syncthreads();
         if (s_take && v.bits) {
+            const uint32_t B = s_B[0];
             for (int wi = tid; wi < v.words; wi += nt) {
                 uint32_t word = 0u;
                 const int v0 = wi * 32, v1 = min(n, v0 + 32);
@@ -409,7 +506,15 @@ int finalize_launch(const FinalArgs &a, void *stream)
 
 int opt_readout_launch(const OptArgs &a, int grid, void *stream)
 {
-    opt_readout_kernel<<<grid, 1024, 0, reinterpret_cast<cudaStream_t>(stream)>>>(a);
+    static SmemLimit shared, global;
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    const size_t hist = (size_t)kDigits * 33 * 4, all = hist + (size_t)a.v.n * 8;
+    if (all <= raise_smem(shared, opt_readout_kernel<true>)) {
+        opt_readout_kernel<true><<<grid, kOptThreads, all, st>>>(a);
+    } else {
+        if (hist > raise_smem(global, opt_readout_kernel<false>)) return -1;
+        opt_readout_kernel<false><<<grid, kOptThreads, hist, st>>>(a);
+    }
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

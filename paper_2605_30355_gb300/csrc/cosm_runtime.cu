@@ -1291,12 +1291,10 @@ int cosm::upload_alpha(cosm_handle *h, int64_t S, cudaStream_t st)
 int cosm::launch_opt_readout(cosm_handle *h, bool keep_better, cudaStream_t st)
 {
     const int n = h->g.n;
-    int npow2 = 1;
-    while (npow2 < n) npow2 <<= 1;
     const int grid = std::max(1, std::min(h->replicas, h->num_sms));
     int rc;
     if ((rc = h->d_qbuf.ensure((size_t)grid * n)) || (rc = h->d_delta.ensure((size_t)grid * n)) ||
-        (rc = h->d_items.ensure((size_t)grid * npow2)))
+        (rc = h->d_items.ensure((size_t)grid * 2 * n)))
         return rc;
     OptArgs o;
     std::memset(&o, 0, sizeof(o));
@@ -1305,7 +1303,6 @@ int cosm::launch_opt_readout(cosm_handle *h, bool keep_better, cudaStream_t st)
     o.qbuf = h->d_qbuf.p;
     o.delta = h->d_delta.p;
     o.items = h->d_items.p;
-    o.npow2 = npow2;
     o.keep_better = keep_better ? 1 : 0;
     o.storage = h->prm.storage;
     if (opt_readout_launch(o, grid, st))
