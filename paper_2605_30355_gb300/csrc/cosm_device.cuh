@@ -73,10 +73,20 @@ __device__ __forceinline__ float rint_fast(float v)
 }
 __device__ __forceinline__ float wrap_c(float v) { return __fadd_rn(v, -rint_fast(v)); }
 
-// q = floor(x 2^32) mod 2^32 of the turn x represented by g (exact).
+// q = floor(x 2^32) mod 2^32 of the turn x represented by g (exact). For |g| <
+// 64 without the 64-bit conversion (an eighth of the others' rate): a = floor(
+// 2^16 g) in the low bits of an FMA rounded toward -inf, the rest b = g - 2^-16
+// a, rounded toward -inf too (multiples of 2^-32 below 2^-16 are representable,
+// so its floor in them is exact), and floor(2^32 b) the same way; the two
+// halves are the low half-words of the FMAs.
 __device__ __forceinline__ uint32_t phase_q(float g)
 {
-    return (uint32_t)(unsigned long long)__float2ll_rd(g * 4294967296.0f);
+    const float t = __fmaf_rd(g, 65536.0f, 12582912.0f);
+    const float b = __fmaf_rd(__fadd_rn(t, -12582912.0f), -0x1p-16f, g);
+    const float l = __fmaf_rd(b, 4294967296.0f, 8388608.0f);
+    uint32_t q = __byte_perm(__float_as_uint(l), __float_as_uint(t), 0x5410);
+    if (!(fabsf(g) < 64.0f)) q = (uint32_t)(unsigned long long)__float2ll_rd(g * 4294967296.0f);
+    return q;
 }
 
 // ---------------------------------------------------------------- checked build
@@ -328,6 +338,7 @@ __device__ __forceinline__ void dwt_apply(float (&x)[K], const float *thc, const
 // one thread per replica on every event's critical path. E = min(32, P)
 // words fit the P + 1 of a replica's array. A barrier separates the fill from
 // the first use, and every use from the next fill (both hold in every sweep).
+// Direction bit k of a replica: the drawn direction of event k.
 template <bool kQ, int K>
 __device__ __noinline__ void twist_fill(const InstView &v, int *D, int E, int stride, bool randdir, uint32_t s,
                                         uint32_t rep0)
@@ -353,26 +364,43 @@ __device__ __noinline__ void twist_fill(const InstView &v, int *D, int E, int st
     }
 }
 
-struct TwistWindow {
-    int left = 0;  // events left in the window
-    int E;
-    int stride;  // sweeps between events
-    bool randdir;
-    __device__ __forceinline__ TwistWindow(const InstView &v, bool on)
-        : E(min(32, v.P)), stride(on ? v.dwt_period : 1), randdir((v.flags & COSM_DWT_RANDOM_DIR) != 0)
+// A segment's sweeps in stretches: one window of twist events, or up to the
+// next tracking readout, whichever ends first. Inside a stretch the sweep loop
+// makes no call, so its registers are its own.
+struct Stretches {
+    bool dwt_on, randdir;
+    uint32_t period, track, S, E;
+    __device__ __forceinline__ Stretches(const InstView &v)
+        : dwt_on(!(v.flags & COSM_NO_DWT) && v.dwt_period > 0), randdir((v.flags & COSM_DWT_RANDOM_DIR) != 0),
+          period((uint32_t)v.dwt_period), track((uint32_t)v.track), S((uint32_t)v.S), E((uint32_t)min(32, v.P))
     {
     }
-    // Index of sweep s's event in the window; refills it when it is used up.
+    // Last sweep of the stretch from s on (at most s1 < 2^31). Fills the window
+    // with the stretch's events; *to_twist: sweeps before the first.
     template <bool kQ, int K>
-    __device__ __forceinline__ int next(const InstView &v, int *D, uint32_t s, uint32_t rep0)
+    __device__ __forceinline__ uint32_t begin(const InstView &v, int *D, uint32_t s, uint32_t s1, uint32_t rep0,
+                                              int *to_twist)
     {
-        if (left == 0) {
-            twist_fill<kQ, K>(v, D, E, stride, randdir, s, rep0);
-            left = E;
+        uint32_t end = s1;
+        if (track > 0) end = min(end, s + (track - 1 - (s - 1) % track));  // the next multiple of track
+        *to_twist = 0x7FFFFFFF;
+        if (dwt_on) {
+            const uint32_t wait = period - 1 - (s - 1) % period;  // to the next multiple of the period
+            *to_twist = (int)wait;
+            const uint64_t covered = (uint64_t)s + wait + (uint64_t)E * period - 1;
+            if (covered < end) end = (uint32_t)covered;
+            twist_fill<kQ, K>(v, D, (int)E, (int)period, randdir, s + wait, rep0);
         }
-        return E - left--;
+        return end;
     }
+    __device__ __forceinline__ bool readout_after(uint32_t s) const { return track > 0 && (s % track == 0 || s == S); }
 };
+
+// Sweeps before the next one that wraps (a multiple of wrap_p; 0: none).
+__device__ __forceinline__ int sweeps_to_wrap(uint32_t s, int wrap_p)
+{
+    return wrap_p > 0 ? wrap_p - 1 - (int)((s - 1) % (uint32_t)wrap_p) : 0x7FFFFFFF;
+}
 
 // ---------------------------------------------------------------- segments
 // Shared-memory layout of one tile and the per-segment prologue (bounded
@@ -411,7 +439,7 @@ __device__ __forceinline__ Tile<Store, K> carve(unsigned char *smem, int n, int 
 
 // Returns false when the bounded wait gave up (the error word is set).
 template <typename Store, int K>
-__device__ bool seg_begin(const InstView &v, const Segment &sg, const Tile<Store, K> &t, int *s_skip,
+__device__ __noinline__ bool seg_begin(const InstView &v, const Segment sg, const Tile<Store, K> t, int *s_skip,
                           int32_t *ready, int32_t *err, uint64_t wait_limit_ns)
 {
     const int tid = threadIdx.x, nt = blockDim.x;
@@ -447,19 +475,24 @@ __device__ bool seg_begin(const InstView &v, const Segment &sg, const Tile<Store
 #endif
     const Store *gst = reinterpret_cast<const Store *>(v.state) + (size_t)sg.tile * v.state_tile_stride;
     if (sg.flags & SEG_INIT) {
-        // Alg. 1 "Set x_i random": Philox keyed by seed, counter (v/4, r, 0, 0)
+        // Alg. 1 "Set x_i random": Philox keyed by seed, counter (v/4, r, 0, 0);
+        // one draw gives four vertices of a replica their phases
         const uint32_t rep0 = (uint32_t)sg.tile * K;
         const uint32_t k0 = (uint32_t)v.seed, k1 = (uint32_t)(v.seed >> 32);
-        for (int k = tid; k < v.n * K; k += nt) {
-            const int slot = k / K, r = k % K;
-            const uint32_t ov = (uint32_t)v.orig_of[slot];
-            uint32_t c[4] = {ov >> 2, rep0 + (uint32_t)r, 0u, 0u};
+        for (int k = tid; k < (v.n + 3) / 4 * K; k += nt) {
+            const int j = k / K, r = k % K;
+            uint32_t c[4] = {(uint32_t)j, rep0 + (uint32_t)r, 0u, 0u};
             philox4x32_10(c, k0, k1);
-            const uint32_t lo = (ov & 1) ? c[1] : c[0], hi = (ov & 1) ? c[3] : c[2];
-            const uint32_t word = (ov & 2) ? hi : lo;
-            if constexpr (std::is_same<Store, uint16_t>::value) t.xs[k] = (uint16_t)(word >> 16);
-            else if constexpr (sizeof(Store) == 4) t.xs[k] = u24_centered(word);
-            else t.xs[k] = to_store<Store>(u24_centered(word));
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int ov = 4 * j + q;
+                if (ov >= v.n) break;
+                const int slot = v.slot_of ? (int)__ldg(v.slot_of + ov) : ov;
+                Store *x = t.xs + slot * K + r;
+                if constexpr (std::is_same<Store, uint16_t>::value) *x = (uint16_t)(c[q] >> 16);
+                else if constexpr (sizeof(Store) == 4) *x = u24_centered(c[q]);
+                else *x = to_store<Store>(u24_centered(c[q]));
+            }
         }
         // mid-anneal tracking keeps the lowest-energy readout of the trial
         if (v.track > 0 && v.energy && tid < K && rep0 + tid < (uint32_t)v.replicas)
@@ -485,7 +518,7 @@ __device__ bool seg_begin(const InstView &v, const Segment &sg, const Tile<Store
 // to trace[k] (k >= 0), and with tracking the spins of a replaced readout
 // are saved as bits.
 template <typename Store, int K>
-__device__ __noinline__ void tile_readout(const InstView &a, int tile, const Tile<Store, K> &t, int k, bool keep_better)
+__device__ __noinline__ void tile_readout(const InstView &a, int tile, const Tile<Store, K> t, int k, bool keep_better)
 {
     const int tid = threadIdx.x, nt = blockDim.x, P = a.P;
     const uint32_t rep0 = (uint32_t)tile * K;
@@ -528,32 +561,42 @@ __device__ __noinline__ void tile_readout(const InstView &a, int tile, const Til
             }
         }
     } else {
+        // four edges' records in flight, then their phases
         int base[K];
 #pragma unroll
         for (int r = 0; r < K; ++r) base[r] = 0;
-        for (int e = tid; e < m; e += nt) {
-            const uint32_t rec = load_rec(a, e);
-            const int wv = (int)__ldg(a.w + e);
-            const int i = (int)(rec & 0xFFFFu), j = (int)(rec >> 16);
-            uint32_t qis[K], qjs[K];
-            ld_q32<Store, K>(t.xs + (size_t)i * K, qis);
-            ld_q32<Store, K>(t.xs + (size_t)j * K, qjs);
+        constexpr int U = 4;
+        for (int e0 = tid; e0 < m; e0 += U * nt) {
+            uint32_t rec[U];
+            int wv[U];
 #pragma unroll
-            for (int r = 0; r < K; ++r) {
-                const uint32_t qi = qis[r], qj = qjs[r];
-                const int fi = (int)(((uint64_t)((qi & 0x7FFFFFFFu) + 1u) * (uint64_t)P + 0x7FFFFFFFull) >> 31);
-                const int fj = (int)(((uint64_t)((qj & 0x7FFFFFFFu) + 1u) * (uint64_t)P + 0x7FFFFFFFull) >> 31);
-                const int lo = min(fi, fj), hi = max(fi, fj);
-                int *Dr = t.D + r * (P + 1);
-                if ((qi >> 31) == (qj >> 31)) {
-                    if (lo < hi) {  // cut for p in [lo, hi)
-                        atomicAdd(Dr + lo, wv);
-                        atomicAdd(Dr + hi, -wv);
+            for (int u = 0; u < U; ++u) {
+                const int e = e0 + u * nt;
+                rec[u] = e < m ? load_rec(a, e) : 0u;
+                wv[u] = e < m ? (int)__ldg(a.w + e) : 0;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (e0 + u * nt >= m) break;
+                uint32_t qis[K], qjs[K];
+                ld_q32<Store, K>(t.xs + (size_t)(rec[u] & 0xFFFFu) * K, qis);
+                ld_q32<Store, K>(t.xs + (size_t)(rec[u] >> 16) * K, qjs);
+#pragma unroll
+                for (int r = 0; r < K; ++r) {
+                    const uint32_t qi = qis[r], qj = qjs[r];
+                    const int fi = (int)(((uint64_t)((qi & 0x7FFFFFFFu) + 1u) * (uint32_t)P + 0x7FFFFFFFull) >> 31);
+                    const int fj = (int)(((uint64_t)((qj & 0x7FFFFFFFu) + 1u) * (uint32_t)P + 0x7FFFFFFFull) >> 31);
+                    const int lo = min(fi, fj), hi = max(fi, fj);
+                    int *Dr = t.D + r * (P + 1);
+                    // same half: cut for p in [lo, hi), else for p in [0, lo)
+                    // and [hi, P) (entry P is never read)
+                    const bool across = ((qi ^ qj) >> 31) != 0;
+                    const int d = across ? -wv[u] : wv[u];
+                    if (across) base[r] += wv[u];
+                    if (lo < hi) {
+                        atomicAdd(Dr + lo, d);
+                        atomicAdd(Dr + hi, -d);
                     }
-                } else {  // cut for p in [0, lo) and [hi, P)
-                    base[r] += wv;
-                    if (lo < P) atomicAdd(Dr + lo, -wv);
-                    if (hi < P) atomicAdd(Dr + hi, wv);
                 }
             }
         }
@@ -566,9 +609,12 @@ __device__ __noinline__ void tile_readout(const InstView &a, int tile, const Til
         }
     }
     __syncthreads();
-    if (tid < K) {
-        const uint32_t rep = rep0 + tid;
-        const int *Dr = t.D + tid * (P + 1);
+    // one warp per replica (whole warps only): the best bisector from the
+    // prefix sums over p, eight entries per lane, ties to the smallest p
+    const int lane = tid & 31, warps = max(1, nt >> 5);
+    for (int rr = tid >> 5; rr < K && (tid >> 5) < warps; rr += warps) {
+        const uint32_t rep = rep0 + rr;
+        const int *Dr = t.D + rr * (P + 1);
         long long cut, F = 0;
         int bp;
         uint32_t B;
@@ -578,30 +624,47 @@ __device__ __noinline__ void tile_readout(const InstView &a, int tile, const Til
             bp = -1;
             B = 0xC0000000u;
         } else {
-            long long accv = 0;
+            const int per = (P + 31) >> 5, p0 = lane * per, p1 = min(P, p0 + per);
+            long long sum = 0;
+            for (int p = p0; p < p1; ++p) sum += Dr[p];
+            long long run = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const long long y = __shfl_up_sync(0xFFFFFFFFu, run, o);
+                if (lane >= o) run += y;
+            }
+            run -= sum;
             cut = LLONG_MIN;
             bp = 0;
-            for (int p = 0; p < P; ++p) {
-                accv += Dr[p];
-                if (accv > cut) { cut = accv; bp = p; }
+            for (int p = p0; p < p1; ++p) {
+                run += Dr[p];
+                if (run > cut) { cut = run; bp = p; }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const long long c = __shfl_xor_sync(0xFFFFFFFFu, cut, o);
+                const int q = __shfl_xor_sync(0xFFFFFFFFu, bp, o);
+                if (c > cut || (c == cut && q < bp)) { cut = c; bp = q; }
             }
             B = (uint32_t)(((uint64_t)bp << 31) / (uint64_t)P);
         }
-        int take = 0;
-        if (rep < (uint32_t)a.replicas) {
-            const long long E = a.W - 2 * cut - F;
-            if (k >= 0 && a.trace) a.trace[(size_t)rep * a.n_trace + k] = E;
-            // __ldcg: the value may come from a segment of this tile run on another SM
-            take = !keep_better || !a.energy || E < __ldcg(a.energy + rep);
-            if (take) {
-                a.cut[rep] = cut;
-                a.bestp[rep] = bp;
-                if (a.energy) a.energy[rep] = E;
-                if (a.bisB) a.bisB[rep] = B;
+        if (lane == 0) {
+            int take = 0;
+            if (rep < (uint32_t)a.replicas) {
+                const long long E = a.W - 2 * cut - F;
+                if (k >= 0 && a.trace) a.trace[(size_t)rep * a.n_trace + k] = E;
+                // __ldcg: the value may come from a segment of this tile run on another SM
+                take = !keep_better || !a.energy || E < __ldcg(a.energy + rep);
+                if (take) {
+                    a.cut[rep] = cut;
+                    a.bestp[rep] = bp;
+                    if (a.energy) a.energy[rep] = E;
+                    if (a.bisB) a.bisB[rep] = B;
+                }
             }
+            t.imp[rr] = take;
+            t.Bs[rr] = B;
         }
-        t.imp[tid] = take;
-        t.Bs[tid] = B;
     }
     if (!a.bits) return;
     __syncthreads();
@@ -632,7 +695,7 @@ __device__ __noinline__ void tile_readout(const InstView &a, int tile, const Til
 }
 
 template <typename Store, int K>
-__device__ void seg_end(const InstView &a, const Segment &sg, const Tile<Store, K> &t, int32_t *ready)
+__device__ __noinline__ void seg_end(const InstView &a, const Segment sg, const Tile<Store, K> t, int32_t *ready)
 {
     const int tid = threadIdx.x, nt = blockDim.x;
     // with tracking the readout after the last sweep ran inside the sweep loop

@@ -359,15 +359,11 @@ __device__ __forceinline__ void run_segment_edges(const InstView &v, const Segme
     const Tile<Store, K> t = carve<Store, K>(edges_smem, v.n, v.P, false);
     const int tid = threadIdx.x, nt = blockDim.x;
     if (!seg_begin<Store, K>(v, sg, t, s_skip, ready, err, wait_limit_ns)) return;
-    const bool dwt_on = !(v.flags & COSM_NO_DWT) && v.dwt_period > 0;
-    const int period = v.dwt_period, track = v.track;
-    const uint32_t wrap_p = (uint32_t)v.wrap_p, rep0 = (uint32_t)sg.tile * K;
-    TwistWindow tw(v, dwt_on);
-    const uint32_t s0 = (uint32_t)sg.s_begin, s1 = (uint32_t)sg.s_end;  // below 2^31
-    if (s0 <= s1) {
-        int phase = dwt_on ? (int)(s0 % (uint32_t)period) : 1;
-        const float2 *ap = v.alpha_tab + (sg.s_begin - v.alpha_base);
-        float2 at = __ldg(ap);
+    Stretches st(v);
+    const uint32_t rep0 = (uint32_t)sg.tile * K;
+    const uint32_t s1 = (uint32_t)sg.s_end;  // below 2^31
+    const int wrap_p = v.wrap_p, period = v.dwt_period;
+    if (sg.s_begin <= sg.s_end) {
         static_assert(B <= kRowsAhead, "rows ahead");
         const uint32_t *const start = v.rec + __ldg(v.starts + (tid >> 5)) + (tid & 31) * RW;
         const int nc = v.n_colours;
@@ -376,8 +372,20 @@ __device__ __forceinline__ void run_segment_edges(const InstView &v, const Segme
         Stream<RW, B> stream;
         stream.p = start;
         stream.fetch();
-        for (uint32_t s = s0; s <= s1; ++s) {
-            const bool dwt = dwt_on && phase == 0;
+        for (uint32_t s = (uint32_t)sg.s_begin; s <= s1;) {
+            int to_twist;
+            const uint32_t end = st.template begin<kQ, K>(v, t.D, s, s1, rep0, &to_twist);
+            int to_wrap = sweeps_to_wrap(s, wrap_p), event = -1;
+            const float2 *ap = v.alpha_tab + ((int64_t)s - v.alpha_base);
+            float2 at = __ldg(ap);
+#pragma unroll 1
+            for (int left = (int)(end - s); left >= 0; --left) {
+            const bool dwt = to_twist == 0;
+            if (dwt) {
+                ++event;
+                to_twist = period;
+            }
+            --to_twist;
             EdgeStep c;
             c.alpha = at.x;
             if constexpr (kQ) {
@@ -386,9 +394,7 @@ __device__ __forceinline__ void run_segment_edges(const InstView &v, const Segme
                 c.nw = both_halves(0u - c.aq);
             }
             const float step = at.y;
-            int event = 0;
-            if (dwt) event = tw.template next<kQ, K>(v, t.D, s, rep0);
-            if (s < s1) at = __ldg(++ap);
+            if (left > 0) at = __ldg(++ap);
             edge_sweep<Store, K, kFmt, kEach>(v, counts, nc, rows, stream, c);
             stream.p = start;  // the rows fetched past the end are the first ones
             if (v.hv) {
@@ -405,7 +411,7 @@ __device__ __forceinline__ void run_segment_edges(const InstView &v, const Segme
                     for (int r = 0; r < K; ++r) {
                         const int *Dr = t.D + r * (v.P + 1);
                         cq[r] = (uint32_t)Dr[event];
-                        sq[r] = ((uint32_t)Dr[tw.E] >> event) & 1u ? 0u - stepq : stepq;
+                        sq[r] = ((uint32_t)Dr[st.E] >> event) & 1u ? 0u - stepq : stepq;
                     }
                     dwt_qw_consts<NW>(cq, v.qwin, sq, chw, ntw, sqw);
                     const uint32_t xb = (uint32_t)__cvta_generic_to_shared(t.xs);
@@ -421,18 +427,20 @@ __device__ __forceinline__ void run_segment_edges(const InstView &v, const Segme
             } else {
                 // binary32 wraps on every wrap_p-th sweep, or with every
                 // twist when each update is wrapped
-                const bool wrap = sizeof(Store) == 4 && (wrap_p == 0 ? dwt : s % wrap_p == 0);
+                const bool wrap = sizeof(Store) == 4 && (kEach ? dwt : to_wrap == 0);
+                if (to_wrap == 0) to_wrap = wrap_p;
+                --to_wrap;
                 if (dwt || wrap) {
-                    edge_twist<Store, K>(v, t, event, tw.E, step, dwt, wrap);
+                    edge_twist<Store, K>(v, t, event, (int)st.E, step, dwt, wrap);
                     __syncthreads();
                 }
             }
-            if (dwt_on && ++phase == period) phase = 0;
-            if (track > 0 && (s % (uint32_t)track == 0 || s == (uint32_t)v.S)) {
-                tile_readout<Store, K>(v, sg.tile, t, (int)((s - 1) / (uint32_t)track), true);
-                __syncthreads();
-                tw.left = 0;  // the readout used the window's memory
             }
+            if (st.readout_after(end)) {
+                tile_readout<Store, K>(v, sg.tile, t, (int)((end - 1) / st.track), true);
+                __syncthreads();
+            }
+            s = end + 1;
         }
     }
     seg_end<Store, K>(v, sg, t, ready);
@@ -440,7 +448,8 @@ __device__ __forceinline__ void run_segment_edges(const InstView &v, const Segme
 
 // One kernel for single runs (segment lists) and queues (batch, serving).
 template <typename Store, int K, int kFmt, bool kEach>
-__global__ void __launch_bounds__(edges_max_threads<Store, K>()) edges_kernel(const KernelArgs a, const BatchArgs b)
+__global__ void __launch_bounds__(edges_max_threads<Store, K>()) edges_kernel(const __grid_constant__ KernelArgs a,
+                                                                                    const __grid_constant__ BatchArgs b)
 {
     __shared__ int s_skip, s_unit;
     if (b.units == nullptr) {

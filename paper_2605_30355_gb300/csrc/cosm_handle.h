@@ -108,6 +108,7 @@ struct cosm_handle {
     const cosm::RecordTable *table = nullptr;  // the current layout's
     int format = -1;                // record-table format of the current layout (-1: none)
     DevBuf<int32_t> d_orig;
+    DevBuf<uint16_t> d_slot;        // original id -> slot (lattices)
     DevBuf<int32_t> d_off;          // colour offsets
     int mode = cosm::MODE_GENERAL_;       // kernel variant
     int32_t Q = 0, Wd = 0;          // 2D lattice geometry

@@ -48,7 +48,8 @@ struct InstView {
     const uint32_t *counts;
     const int32_t *starts;
     int32_t n_colours;
-    const int32_t *orig_of;  // slot -> original vertex id (Philox init key)
+    const int32_t *orig_of;  // slot -> original vertex id
+    const uint16_t *slot_of; // original vertex id -> slot, nullptr: the same
     // 2D lattice mode: Q = n/4 slots per sublattice, Wd = L2/2 columns;
     // wnib[pass * Q + f] holds the weight bits of the four edges of 2x2
     // block f in that pass (bit set: w = -1)

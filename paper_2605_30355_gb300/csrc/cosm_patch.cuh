@@ -485,55 +485,65 @@ __device__ __forceinline__ void run_segment_patch(const InstView &v, const Segme
         p.template tile<true>(xs, v, br0, bc0);
     }
     __syncthreads();  // the published sites take the place of the tile
-    const bool dwt_on = !(v.flags & COSM_NO_DWT) && v.dwt_period > 0;
-    const int period = v.dwt_period, wrap_p = v.wrap_p, track = v.track;
-    TwistWindow tw(v, dwt_on);
+    Stretches st(v);
     const uint32_t rep0 = (uint32_t)sg.tile * K;
+    const uint32_t s1 = (uint32_t)sg.s_end;  // below 2^31
+    const int wrap_p = sizeof(Store) == 2 ? 1 : max(v.wrap_p, 1);
     SweepConsts c;
     c.D = t.D;
-    c.E = tw.E;
+    c.E = (int)st.E;
     c.P1 = v.P + 1;
     c.W2 = 2.0f * v.window;
     c.qwin = v.qwin;
-    c.k = 0;
-    const uint32_t s0 = (uint32_t)sg.s_begin, s1 = (uint32_t)sg.s_end;  // below 2^31
-    int phase = dwt_on ? (int)(s0 % (uint32_t)period) : 1;
-    const float2 *ap = v.alpha_tab + (sg.s_begin - v.alpha_base);
-    float2 at = __ldg(ap);
-    for (uint32_t s = s0; s <= s1; ++s) {
-        c.dwt = dwt_on && phase == 0;
-        c.wrap = sizeof(Store) == 2 || wrap_p <= 1 || s % (uint32_t)wrap_p == 0;
-        if constexpr (kQ) {
-            const uint32_t aq = (uint32_t)__float2int_rn(at.x);
-            c.a1 = both_halves(aq);
-            c.n1 = both_halves(0u - aq);
-        } else {
-            c.a1 = __float_as_uint(at.x);
+    for (uint32_t s = (uint32_t)sg.s_begin; s <= s1;) {
+        int to_twist;
+        const uint32_t end = st.template begin<kQ, K>(v, t.D, s, s1, rep0, &to_twist);
+        int to_wrap = sweeps_to_wrap(s, wrap_p);
+        const float2 *ap = v.alpha_tab + ((int64_t)s - v.alpha_base);
+        float2 at = __ldg(ap);
+        const int period = (int)st.period;
+        c.k = -1;
+#pragma unroll 1
+        for (int left = (int)(end - s); left >= 0; --left) {
+            c.dwt = to_twist == 0;
+            c.wrap = to_wrap == 0;
+            if (c.dwt) {
+                ++c.k;
+                to_twist = period;
+            }
+            if (c.wrap) to_wrap = wrap_p;
+            --to_twist;
+            --to_wrap;
+            if constexpr (kQ) {
+                const uint32_t aq = (uint32_t)__float2int_rn(at.x);
+                c.a1 = both_halves(aq);
+                c.n1 = both_halves(0u - aq);
+            } else {
+                c.a1 = __float_as_uint(at.x);
+            }
+            c.step = at.y;
+            if (left > 0) at = __ldg(++ap);
+            if (active) {
+                p.template evens<true>(c);
+                p.template evens<false>(c);
+                p.publish();
+            }
+            __syncthreads();
+            if (active) {
+                p.borrow();
+                p.odd_pass(c);
+                p.give_back();
+            }
+            __syncthreads();
+            if (active) p.take_back();
         }
-        c.step = at.y;
-        if (c.dwt) c.k = tw.template next<kQ, K>(v, t.D, s, rep0);
-        if (s < s1) at = __ldg(++ap);
-        if (active) {
-            p.template evens<true>(c);
-            p.template evens<false>(c);
-            p.publish();
-        }
-        __syncthreads();
-        if (active) {
-            p.borrow();
-            p.odd_pass(c);
-            p.give_back();
-        }
-        __syncthreads();
-        if (active) p.take_back();
-        if (dwt_on && ++phase == period) phase = 0;
-        if (track > 0 && (s % (uint32_t)track == 0 || s == (uint32_t)v.S)) {
+        if (st.readout_after(end)) {
             __syncthreads();  // the tile takes the place of the published sites
             if (active) p.template tile<false>(xs, v, br0, bc0);
-            tile_readout<Store, K>(v, sg.tile, t, (int)((s - 1) / (uint32_t)track), true);
+            tile_readout<Store, K>(v, sg.tile, t, (int)((end - 1) / st.track), true);
             __syncthreads();
-            tw.left = 0;  // the readout used the window's memory
         }
+        s = end + 1;
     }
     __syncthreads();
     if (active) p.template tile<false>(xs, v, br0, bc0);

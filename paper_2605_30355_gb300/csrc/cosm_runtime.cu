@@ -134,7 +134,7 @@ extern "C" void cosm_destroy(cosm_handle *h)
 {
     if (!h) return;
     if (h->stream || h->have_state) cudaStreamSynchronize(h->stream);
-    h->d_ij.release(); h->d_w.release(); h->d_ijs.release(); h->d_orig.release(); h->d_off.release(); h->d_state.release();
+    h->d_ij.release(); h->d_w.release(); h->d_ijs.release(); h->d_orig.release(); h->d_slot.release(); h->d_off.release(); h->d_state.release();
     h->d_cut.release(); h->d_bestp.release(); h->d_alpha.release(); h->d_segs.release();
     h->d_segoff.release(); h->d_ready.release(); h->d_err.release(); h->d_best.release();
     h->d_spins.release();
@@ -438,6 +438,17 @@ extern "C" int cosm_create(const cosm_graph_desc *gd, const cosm_params *p, cosm
         cudaMemset(h->d_err.p, 0, 4) != cudaSuccess) {
         cosm_destroy(h);
         return fail(COSM_ERR_CUDA, "copying the graph to the device failed");
+    }
+    if (h->lattice) {
+        std::vector<uint16_t> slots(h->slot_of.begin(), h->slot_of.end());
+        if ((rc = h->d_slot.ensure(slots.size()))) {
+            cosm_destroy(h);
+            return rc;
+        }
+        if (cudaMemcpy(h->d_slot.p, slots.data(), slots.size() * 2, cudaMemcpyHostToDevice) != cudaSuccess) {
+            cosm_destroy(h);
+            return fail(COSM_ERR_CUDA, "copying the graph to the device failed");
+        }
     }
     // +-1 weights on at most 2^15 slots: the weight folded into the record
     bool unit = g.n <= (1 << 15);
@@ -1122,6 +1133,7 @@ InstView cosm::inst_view(cosm_handle *h)
     // test hook: COSM_SPLIT_W keeps the split records and weights
     v.ijs = std::getenv("COSM_SPLIT_W") ? nullptr : h->d_ijs.p;
     v.orig_of = h->d_orig.p;
+    v.slot_of = h->d_slot.p;
     v.wnib = h->d_wnib.p;
     v.Q = h->Q;
     v.Wd = h->Wd;
