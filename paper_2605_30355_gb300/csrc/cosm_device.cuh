@@ -2053,36 +2053,38 @@ enum { MODE_GENERAL = 0, MODE_ACCUM = 1, MODE_LATTICE2D = 2 };
 // s = +1 iff the minimum angular difference of x_v from 0 is >= 0. Each
 // vertex appears once, so the field updates form one more conflict-free
 // sub-sweep, after the colours.
+// The pass walks the list of slots that have one (1,000 of 10,000 vertices:
+// one step per thread instead of ten, nine of them skipped).
 template <typename Store, int K>
 __device__ __forceinline__ void field_pass(const InstView &a, Store *xs, float alpha)
 {
-    for (int u = threadIdx.x; u < a.n; u += blockDim.x) {
-        const int hvu = __ldg(a.hv + u);
-        if (hvu == 0) continue;
-        const float aw = alpha * (float)(-hvu);
+    for (int k = threadIdx.x; k < a.n_fields; k += blockDim.x) {
+        const int2 f = __ldg(a.hlist + k);
+        const float aw = alpha * (float)(-f.y);
+        Store *p = xs + f.x * K;
         float x[K];
-        ldk<K>(xs + (size_t)u * K, x);
+        ldk<K>(p, x);
 #pragma unroll
         for (int r = 0; r < K; ++r) {
             const float st = floor_parity(2.0f, x[r]) ? -aw : aw;
             x[r] = wrap_c(__fadd_rn(x[r], st));
         }
-        stk<K>(xs + (size_t)u * K, x);
+        stk<K>(p, x);
     }
 }
 
 template <int K>
 __device__ __forceinline__ void field_pass_q(const InstView &a, uint16_t *xs, uint32_t aq)
 {
-    for (int u = threadIdx.x; u < a.n; u += blockDim.x) {
-        const int hvu = __ldg(a.hv + u);
-        if (hvu == 0) continue;
-        const uint32_t ap = (aq * (uint32_t)(-hvu)) << 16;
+    for (int k = threadIdx.x; k < a.n_fields; k += blockDim.x) {
+        const int2 f = __ldg(a.hlist + k);
+        const uint32_t ap = (aq * (uint32_t)(-f.y)) << 16;
+        uint16_t *p = xs + f.x * K;
         uint32_t x[K];
-        ldq<K>(xs + (size_t)u * K, x);
+        ldq<K>(p, x);
 #pragma unroll
         for (int r = 0; r < K; ++r) x[r] += ((int32_t)x[r] >= 0) ? ap : 0u - ap;
-        stq<K>(xs + (size_t)u * K, x);
+        stq<K>(p, x);
     }
 }
 

@@ -119,6 +119,8 @@ struct cosm_handle {
     DevBuf<uint32_t> d_pwt[cosm::kPatchShapes];
     bool fields = false;            // local fields given
     DevBuf<int32_t> d_h;            // local field per slot
+    DevBuf<int2> d_hlist;           // (slot, field) of the vertices with one
+    int32_t n_fields = 0;
     // per run
     DevBuf<unsigned char> d_state;
     DevBuf<int64_t> d_cut;

@@ -81,6 +81,8 @@ struct InstView {
     int32_t *bestp;       // [replicas] its bisector index (-1: not an equally spaced one)
     // local fields and readout bookkeeping (nullptr / 0 where unused)
     const int32_t *hv;    // [n] local field per slot (eq. (1)), nullptr = none
+    const int2 *hlist;    // (slot, field) of the n_fields slots with a field
+    int32_t n_fields;
     int64_t W;            // total Max-Cut weight
     int64_t *energy;      // [replicas] energy (eq. (1)) of the kept readout
     uint32_t *bisB;       // [replicas] position of its bisector (2^-32 turn)

@@ -141,7 +141,7 @@ extern "C" void cosm_destroy(cosm_handle *h)
     h->d_wnib.release();
     for (auto &b : h->d_pwt) b.release();
     for (auto &t : h->tables) t->release();
-    h->d_h.release(); h->d_energy.release(); h->d_bisB.release(); h->d_trace.release();
+    h->d_h.release(); h->d_hlist.release(); h->d_energy.release(); h->d_bisB.release(); h->d_trace.release();
     h->d_bits.release(); h->d_qbuf.release(); h->d_delta.release(); h->d_items.release(); h->d_stage.release();
     delete h;
 }
@@ -469,11 +469,18 @@ extern "C" int cosm_create(const cosm_graph_desc *gd, const cosm_params *p, cosm
     if (h->fields) {
         std::vector<int32_t> hs((size_t)g.n);
         for (int32_t v = 0; v < g.n; ++v) hs[(size_t)h->slot_of[(size_t)v]] = gd->h[v];
-        if ((rc = h->d_h.ensure((size_t)g.n))) {
+        // the vertices with a field, as (slot, field) pairs for the sweeps
+        std::vector<int2> list;
+        for (int32_t v = 0; v < g.n; ++v)
+            if (hs[(size_t)v]) list.push_back(make_int2(v, hs[(size_t)v]));
+        h->n_fields = (int32_t)list.size();
+        if ((rc = h->d_h.ensure((size_t)g.n)) || (rc = h->d_hlist.ensure(list.size()))) {
             cosm_destroy(h);
             return rc;
         }
-        if (cudaMemcpy(h->d_h.p, hs.data(), hs.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess) {
+        if (cudaMemcpy(h->d_h.p, hs.data(), hs.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
+            (!list.empty() && cudaMemcpy(h->d_hlist.p, list.data(), list.size() * sizeof(int2),
+                                         cudaMemcpyHostToDevice) != cudaSuccess)) {
             cosm_destroy(h);
             return fail(COSM_ERR_CUDA, "copying the local fields to the device failed");
         }
@@ -1164,6 +1171,8 @@ InstView cosm::inst_view(cosm_handle *h)
     v.cut = h->d_cut.p;
     v.bestp = h->d_bestp.p;
     v.hv = h->fields ? h->d_h.p : nullptr;
+    v.hlist = h->d_hlist.p;
+    v.n_fields = h->n_fields;
     v.W = h->W;
     v.energy = h->d_energy.p;
     v.bisB = h->d_bisB.p;
@@ -1898,18 +1907,23 @@ extern "C" int cosm_batch_create(int32_t count, const cosm_graph_desc *graphs, c
 }
 
 // Tile layout of one instance inside a batch. Policy 0: the single-instance
-// rule (choose_layout) scored as if the run filled every CTA slot, since the
-// batch as a whole does: the tile keeping the most replicas resident per SM,
-// ties to the wider tile (one edge record and one barrier serve more
-// replicas). Policy 1: the narrowest tile of the storage type. Policy 2: the
-// single-instance rule with the instance's own replica count. Policy 3: as
-// policy 0 with ties to the narrower tile (more CTAs per SM, whose barriers
-// and record loads overlap).
-static int batch_instance_layout(cosm_batch *b, cosm_handle *h, int32_t replicas)
+// rule (choose_layout) for `fill` replicas, 0.6 of the number of this
+// instance's trials that would be as much work as the whole batch: a batch
+// that fills the GPU takes the tiles that keep it busiest, a small one the
+// tiles that finish a trial soonest (100 sweeps of 16 tori and graphs of 800
+// to 3,000 vertices: 2.2 ms at the whole fill, 1.5 at 0.6, 1.4 at 0.35; 48 of
+// up to 20,000: 9.0 / 8.7 / 9.1). Policy 1: the narrowest tile of the storage
+// type. Policy 2: the single-instance rule with the instance's own replica
+// count. Policy 3: as policy 0 with ties to the narrower tile (more CTAs per
+// SM, whose barriers and record loads overlap). Kernels without a fitted cost
+// (plain records, lattices on shared memory) score policies 0, 1 and 3 as if
+// the run filled every CTA slot.
+static int batch_instance_layout(cosm_batch *b, cosm_handle *h, int32_t replicas, int32_t fill)
 {
     int rc;
     if (b->policy == 2) return choose_layout(h, replicas);
-    if ((rc = choose_layout(h, 1 << 23, b->policy == 3))) return rc;
+    if ((rc = choose_layout(h, fill, b->policy == 3))) return rc;
+    if (h->shape < 0 && h->format < 0 && (rc = choose_layout(h, 1 << 23, b->policy == 3))) return rc;
     if (b->policy == 1 && h->shape < 0 && h->K != (h->prm.storage == COSM_F32 ? 1 : 2)) {
         const int Kmin = h->prm.storage == COSM_F32 ? 1 : 2;
         const size_t esz = h->prm.storage == COSM_F32 ? 4 : 2;
@@ -1981,12 +1995,19 @@ static int batch_layout(cosm_batch *b, const int64_t *sweeps, const int32_t *rep
     const int n = (int)b->hs.size();
     std::vector<InstView> views((size_t)n);
     std::vector<BatchFinal> fins((size_t)n);
+    double total = 0.0;  // edge updates of the run
+    for (int i = 0; i < n; ++i)
+        if (sweeps[i] > 0 && replicas[i] > 0)
+            total += (double)b->hs[(size_t)i]->g.m * (double)replicas[i] * (double)sweeps[i];
     for (int i = 0; i < n; ++i) {
         cosm_handle *h = b->hs[(size_t)i];
         if (sweeps[i] < 1 || sweeps[i] >= ((int64_t)1 << 31) || replicas[i] < 1 || replicas[i] >= (1 << 24))
             return fail(COSM_ERR_INVALID_ARG, "instance " + std::to_string(i) + ": bad sweeps or replicas");
         int rc;
-        if ((rc = batch_instance_layout(b, h, replicas[i]))) return rc;
+        const double fill = 0.6 * total / ((double)h->g.m * (double)sweeps[i]);
+        if ((rc = batch_instance_layout(b, h, replicas[i], (int32_t)std::max((double)replicas[i],
+                                                                            std::min(fill, 8388608.0)))))
+            return rc;
         if (b->threads && h->shape < 0) {
             h->threads = b->threads;
             while (h->threads > 64 && kernel_occupancy(h, h->threads, h->smem, true) == 0)
