@@ -21,7 +21,7 @@ int validate_graph(const Graph &g, std::string &why)
         why = "m must be in [1, 2^26]";
         return COSM_ERR_INVALID_ARG;
     }
-    std::vector<int64_t> key((size_t)g.m);
+    std::vector<int32_t> end((size_t)g.n + 1, 0);
     int64_t abs_sum = 0;
     for (int64_t e = 0; e < g.m; ++e) {
         int32_t a = g.src[(size_t)e], b = g.dst[(size_t)e], wt = g.w[(size_t)e];
@@ -34,17 +34,25 @@ int validate_graph(const Graph &g, std::string &why)
             return COSM_ERR_INVALID_ARG;
         }
         abs_sum += std::abs(wt);
-        key[(size_t)e] = (int64_t)a * g.n + b;
+        ++end[(size_t)a + 1];
     }
     if (abs_sum >= ((int64_t)1 << 31)) {
         why = "sum of |w| must be below 2^31";
         return COSM_ERR_INVALID_ARG;
     }
-    std::sort(key.begin(), key.end());
-    for (size_t e = 1; e < key.size(); ++e)
-        if (key[e] == key[e - 1]) {
-            why = "duplicate edge";
-            return COSM_ERR_INVALID_ARG;
+    // duplicates: each source's destinations, stamped as they are met (linear
+    // in the edges, where sorting the pairs was not)
+    for (int32_t v = 0; v < g.n; ++v) end[(size_t)v + 1] += end[(size_t)v];
+    std::vector<int32_t> by_src((size_t)g.m), stamp((size_t)g.n, -1);
+    for (int64_t e = 0; e < g.m; ++e) by_src[(size_t)end[(size_t)g.src[(size_t)e]]++] = g.dst[(size_t)e];
+    for (int32_t a = 0, k = 0; a < g.n; ++a)
+        for (; k < end[(size_t)a]; ++k) {
+            int32_t &seen = stamp[(size_t)by_src[(size_t)k]];
+            if (seen == a) {
+                why = "duplicate edge";
+                return COSM_ERR_INVALID_ARG;
+            }
+            seen = a;
         }
     return COSM_OK;
 }
@@ -202,6 +210,12 @@ int color_misra_gries(int32_t n, int64_t m, const int32_t *src, const int32_t *d
     return COSM_OK;
 }
 
+// (x + 1) mod L, dividing only where x is no coordinate
+static inline int32_t next_on(int32_t x, int32_t L)
+{
+    return (uint32_t)(x + 1) < (uint32_t)L ? x + 1 : (x + 1) % L;
+}
+
 int color_torus2d(int32_t L1, int32_t L2, int64_t m, const int32_t *src, const int32_t *dst,
                   int32_t *color)
 {
@@ -212,10 +226,10 @@ int color_torus2d(int32_t L1, int32_t L2, int64_t m, const int32_t *src, const i
         const int32_t ra = a / L2, ca = a % L2, rb = b / L2, cb = b % L2;
         // order: even-column horizontal, even-row vertical, odd-column
         // horizontal, odd-row vertical (consecutive pairs act on 2x2 blocks)
-        if (ra == rb && (ca + 1) % L2 == cb) color[e] = (ca & 1) ? 2 : 0;
-        else if (ra == rb && (cb + 1) % L2 == ca) color[e] = (cb & 1) ? 2 : 0;
-        else if (ca == cb && (ra + 1) % L1 == rb) color[e] = (ra & 1) ? 3 : 1;
-        else if (ca == cb && (rb + 1) % L1 == ra) color[e] = (rb & 1) ? 3 : 1;
+        if (ra == rb && next_on(ca, L2) == cb) color[e] = (ca & 1) ? 2 : 0;
+        else if (ra == rb && next_on(cb, L2) == ca) color[e] = (cb & 1) ? 2 : 0;
+        else if (ca == cb && next_on(ra, L1) == rb) color[e] = (ra & 1) ? 3 : 1;
+        else if (ca == cb && next_on(rb, L1) == ra) color[e] = (rb & 1) ? 3 : 1;
         else return COSM_ERR_INVALID_ARG;
     }
     return COSM_OK;
@@ -243,8 +257,8 @@ int color_torus3d(int32_t L1, int32_t L2, int32_t L3, int64_t m, const int32_t *
                 if (b != a && co[0][b] != co[1][b]) same = false;
             if (!same) continue;
             // all even classes (axes 0, 1, 2), then all odd classes
-            if ((co[0][a] + 1) % L[a] == co[1][a]) c = 3 * (co[0][a] & 1) + a;
-            else if ((co[1][a] + 1) % L[a] == co[0][a]) c = 3 * (co[1][a] & 1) + a;
+            if (next_on(co[0][a], L[a]) == co[1][a]) c = 3 * (co[0][a] & 1) + a;
+            else if (next_on(co[1][a], L[a]) == co[0][a]) c = 3 * (co[1][a] & 1) + a;
         }
         if (c < 0) return COSM_ERR_INVALID_ARG;
         color[e] = c;
@@ -256,30 +270,30 @@ int color_torus3d(int32_t L1, int32_t L2, int32_t L3, int64_t m, const int32_t *
 // coordinate, row-major inside a group. In the regular colouring every
 // colour then pairs slot f of one group with slot f (or f + 1, f + row) of
 // another, so consecutive threads touch consecutive shared-memory words.
-bool lattice_relabel(const Graph &g, std::vector<int32_t> &slot_of, std::string &why)
+// pattern receives the lattice's own colouring.
+bool lattice_relabel(const Graph &g, std::vector<int32_t> &slot_of, std::vector<int32_t> &pattern, std::string &why)
 {
     const int32_t *d = g.dims;
-    std::vector<int32_t> col((size_t)g.m);
+    pattern.assign((size_t)g.m, 0);
     slot_of.assign((size_t)g.n, 0);
     if (d[0] > 0 && d[1] > 0 && d[2] == 0) {
         const int32_t L1 = d[0], L2 = d[1];
         // any subset of the torus edges (e.g. couplings that cancelled to 0)
         if ((int64_t)L1 * L2 != g.n || g.m > 2 * (int64_t)g.n ||
-            color_torus2d(L1, L2, g.m, g.src.data(), g.dst.data(), col.data()) != COSM_OK) {
+            color_torus2d(L1, L2, g.m, g.src.data(), g.dst.data(), pattern.data()) != COSM_OK) {
             why = "dims does not describe this graph as an even-sided 2D torus";
             return false;
         }
         const int32_t q = g.n / 4, hw = L2 / 2;
-        for (int32_t v = 0; v < g.n; ++v) {
-            int32_t r = v / L2, c = v % L2;
-            slot_of[(size_t)v] = ((r & 1) * 2 + (c & 1)) * q + (r >> 1) * hw + (c >> 1);
-        }
+        for (int32_t r = 0, v = 0; r < L1; ++r)
+            for (int32_t c = 0; c < L2; ++c, ++v)
+                slot_of[(size_t)v] = ((r & 1) * 2 + (c & 1)) * q + (r >> 1) * hw + (c >> 1);
         return true;
     }
     if (d[0] > 0 && d[1] > 0 && d[2] > 0) {
         const int32_t L1 = d[0], L2 = d[1], L3 = d[2];
         if ((int64_t)L1 * L2 * L3 != g.n || g.m > 3 * (int64_t)g.n ||
-            color_torus3d(L1, L2, L3, g.m, g.src.data(), g.dst.data(), col.data()) != COSM_OK) {
+            color_torus3d(L1, L2, L3, g.m, g.src.data(), g.dst.data(), pattern.data()) != COSM_OK) {
             why = "dims does not describe this graph as an even-sided 3D torus";
             return false;
         }

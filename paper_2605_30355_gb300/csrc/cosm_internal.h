@@ -263,6 +263,6 @@ int color_torus2d(int32_t L1, int32_t L2, int64_t m, const int32_t *src, const i
 int color_torus3d(int32_t L1, int32_t L2, int32_t L3, int64_t m, const int32_t *src,
                   const int32_t *dst, int32_t *color);
 // Vertex -> slot relabel for shared-memory locality (lattice sublattices).
-bool lattice_relabel(const Graph &g, std::vector<int32_t> &slot_of, std::string &why);
+bool lattice_relabel(const Graph &g, std::vector<int32_t> &slot_of, std::vector<int32_t> &pattern, std::string &why);
 
 }  // namespace cosm

@@ -6,7 +6,6 @@
 
 #include <algorithm>
 #include <cmath>
-#include <unordered_map>
 #include <cstdlib>
 #include <cstring>
 #include <string>
@@ -152,7 +151,7 @@ extern "C" void cosm_destroy(cosm_handle *h)
 // passes; this builds each block's four weight bits from the edge list, in
 // the kernel's edge order (even pass: A-B, C-D, A-C, B-D; odd pass: D-C,
 // B-A, D-B, C-A over the shifted block).
-static int setup_lattice2d(cosm_handle *h)
+static int setup_lattice2d(cosm_handle *h, const std::vector<int32_t> &pattern)
 {
     const Graph &g = h->g;
     h->mode = (h->prm.flags & COSM_NO_SCS) ? MODE_ACCUM_ : MODE_GENERAL_;
@@ -162,19 +161,23 @@ static int setup_lattice2d(cosm_handle *h)
         return COSM_OK;
     for (int64_t e = 0; e < g.m; ++e)
         if (g.w[(size_t)e] != 1 && g.w[(size_t)e] != -1) return COSM_OK;
-    std::vector<int32_t> pat((size_t)g.m);
-    if (color_torus2d(g.dims[0], g.dims[1], g.m, g.src.data(), g.dst.data(), pat.data()) != 0)
-        return COSM_OK;
-    if (pat != g.color) return COSM_OK;  // another colour order changes the dynamics
+    if (pattern != g.color) return COSM_OK;  // another colour order changes the dynamics
     const int32_t Q = g.n / 4, Wd = g.dims[1] / 2;
-    std::unordered_map<int64_t, int32_t> wmap;
-    wmap.reserve((size_t)g.m * 2);
-    for (int64_t e = 0; e < g.m; ++e)
-        wmap[(int64_t)g.src[(size_t)e] * g.n + g.dst[(size_t)e]] = g.w[(size_t)e];
-    auto weight = [&](int32_t slot_a, int32_t slot_b) {
-        const int32_t a = h->orig_of[(size_t)slot_a], b = h->orig_of[(size_t)slot_b];
-        auto it = wmap.find((int64_t)std::min(a, b) * g.n + std::max(a, b));
-        return it == wmap.end() ? 0 : it->second;
+    // a slot's edge of each colour: the other end and the weight (a vertex
+    // of the torus has one edge of each of the four colours)
+    std::vector<int32_t> other((size_t)g.n * 4, -1);
+    std::vector<int8_t> wt((size_t)g.n * 4);
+    for (int64_t e = 0; e < g.m; ++e) {
+        const int32_t a = h->slot_of[(size_t)g.src[(size_t)e]], b = h->slot_of[(size_t)g.dst[(size_t)e]];
+        const size_t ka = (size_t)a * 4 + g.color[(size_t)e], kb = (size_t)b * 4 + g.color[(size_t)e];
+        other[ka] = b;
+        other[kb] = a;
+        wt[ka] = wt[kb] = (int8_t)g.w[(size_t)e];
+    }
+    auto weight = [&](int32_t slot_a, int32_t slot_b) -> int32_t {
+        for (size_t k = (size_t)slot_a * 4; k < (size_t)slot_a * 4 + 4; ++k)
+            if (other[k] == slot_b) return wt[k];
+        return 0;
     };
     std::vector<uint8_t> nib((size_t)2 * Q, 0);
     for (int32_t f = 0; f < Q; ++f) {
@@ -363,8 +366,9 @@ extern "C" int cosm_create(const cosm_graph_desc *gd, const cosm_params *p, cosm
     h->C = g.C;
     // shared-memory layout: lattice sublattices when the hint matches
     h->slot_of.resize((size_t)g.n);
+    std::vector<int32_t> pattern;
     if (g.dims[0] > 0) {
-        if (!lattice_relabel(g, h->slot_of, why)) { delete h; return fail(COSM_ERR_INVALID_ARG, why); }
+        if (!lattice_relabel(g, h->slot_of, pattern, why)) { delete h; return fail(COSM_ERR_INVALID_ARG, why); }
         h->lattice = true;
     } else {
         for (int32_t v = 0; v < g.n; ++v) h->slot_of[(size_t)v] = v;
@@ -372,12 +376,21 @@ extern "C" int cosm_create(const cosm_graph_desc *gd, const cosm_params *p, cosm
     h->orig_of.assign((size_t)g.n, 0);
     for (int32_t v = 0; v < g.n; ++v) h->orig_of[(size_t)h->slot_of[(size_t)v]] = v;
     // colour-major edge records, each colour sorted by the slot of src
+    // (stable counting sorts by slot, then by colour: comparing edges through
+    // their indices was half of creating a 100 x 100 instance)
     std::vector<int64_t> order((size_t)g.m);
-    for (int64_t e = 0; e < g.m; ++e) order[(size_t)e] = e;
-    std::stable_sort(order.begin(), order.end(), [&](int64_t a, int64_t b) {
-        if (g.color[(size_t)a] != g.color[(size_t)b]) return g.color[(size_t)a] < g.color[(size_t)b];
-        return h->slot_of[(size_t)g.src[(size_t)a]] < h->slot_of[(size_t)g.src[(size_t)b]];
-    });
+    {
+        std::vector<int64_t> by_slot((size_t)g.m);
+        std::vector<int64_t> at((size_t)std::max(g.n, g.C) + 1, 0);
+        for (int64_t e = 0; e < g.m; ++e) ++at[(size_t)h->slot_of[(size_t)g.src[(size_t)e]] + 1];
+        for (int32_t v = 0; v < g.n; ++v) at[(size_t)v + 1] += at[(size_t)v];
+        for (int64_t e = 0; e < g.m; ++e)
+            by_slot[(size_t)at[(size_t)h->slot_of[(size_t)g.src[(size_t)e]]]++] = e;
+        std::fill(at.begin(), at.end(), 0);
+        for (int64_t e = 0; e < g.m; ++e) ++at[(size_t)g.color[(size_t)e] + 1];
+        for (int32_t c = 0; c < g.C; ++c) at[(size_t)c + 1] += at[(size_t)c];
+        for (int64_t e : by_slot) order[(size_t)at[(size_t)g.color[(size_t)e]]++] = e;
+    }
     // instances that never take record tables (whose rows are arranged for
     // their own tile width) have their colours' edges ordered here
     int32_t wmax = 0;
@@ -485,7 +498,7 @@ extern "C" int cosm_create(const cosm_graph_desc *gd, const cosm_params *p, cosm
             return fail(COSM_ERR_CUDA, "copying the local fields to the device failed");
         }
     }
-    if ((rc = setup_lattice2d(h))) {
+    if ((rc = setup_lattice2d(h, pattern))) {
         cosm_destroy(h);
         return rc;
     }
