@@ -109,18 +109,6 @@ __device__ __forceinline__ uint32_t checked_rec(const InstView &a, uint32_t rec)
     return rec;
 }
 __device__ __forceinline__ uint32_t load_rec(const InstView &a, int e) { return checked_rec(a, __ldg(a.ij + e)); }
-// A record of a.ijs ([w = -1] | slot(src) << 1 | slot(dst) << 16).
-__device__ __forceinline__ uint32_t load_rec_sgn(const InstView &a, int e)
-{
-    const uint32_t rec = __ldg(a.ijs + e);
-#ifdef COSM_CHECKS
-    if (((rec & 0xFFFFu) >> 1) >= (uint32_t)a.n || (rec >> 16) >= (uint32_t)a.n) {
-        if (a.check) atomicOr(a.check, 2);
-        return 0u;
-    }
-#endif
-    return rec;
-}
 
 // ---------------------------------------------------------------- storage
 template <int K>
@@ -1313,14 +1301,10 @@ __device__ __forceinline__ f32x2 p_pack(float lo, float hi)
 // may run past the end e1 of its colour (loads of slot 0, stores skipped).
 // kStaged: the colour's records sit in shared memory (edge e's record at
 // sij + 4 e, its weight at sw + e), else they are read from global memory.
-// kSgn: the records of a.ijs, whose bit 0 is the sign of a +-1 weight, so
-// alpha w is alpha + bit 0 * 2^31 in integer arithmetic (the sign bit
-// flipped; no weight load or conversion).
-template <int K, int B, bool kWrapEach, bool kTail, bool kStaged = false, bool kSgn = false>
+template <int K, int B, bool kWrapEach, bool kTail, bool kStaged = false>
 __device__ __forceinline__ void edge_batch_x2(const InstView &a, uint32_t xb, float alpha, int e0, int e1, int nt,
                                               uint32_t sij = 0, uint32_t sw = 0)
 {
-    static_assert(!(kStaged && kSgn), "staged records carry their weights apart");
     constexpr uint32_t E = K * 4;  // bytes per slot
     uint32_t ai[B], aj[B];
     float aw[B];
@@ -1334,21 +1318,14 @@ __device__ __forceinline__ void edge_batch_x2(const InstView &a, uint32_t xb, fl
                 asm volatile("ld.shared.b32 %0, [%1];" : "=r"(rec) : "r"(sij + 4u * (uint32_t)e) : "memory");
                 asm volatile("ld.shared.s8 %0, [%1];" : "=r"(w) : "r"(sw + (uint32_t)e) : "memory");
                 rec = checked_rec(a, rec);
-            } else if constexpr (kSgn) {
-                rec = load_rec_sgn(a, e);
             } else {
                 rec = load_rec(a, e);
                 w = __ldg(a.w + e);
             }
         }
         aj[u] = xb + (rec >> 16) * E;
-        if constexpr (kSgn) {
-            ai[u] = xb + (rec & 0xFFFEu) * (E / 2);
-            aw[u] = __uint_as_float(flip_if_odd(__float_as_uint(alpha), rec));
-        } else {
-            ai[u] = xb + (rec & 0xFFFFu) * E;
-            aw[u] = alpha * weight_f((int8_t)w);
-        }
+        ai[u] = xb + (rec & 0xFFFFu) * E;
+        aw[u] = alpha * weight_f((int8_t)w);
     }
     if constexpr (K == 1) {
         float xi[B], xj[B];
@@ -1410,7 +1387,7 @@ __device__ __forceinline__ void edge_batch_x2(const InstView &a, uint32_t xb, fl
 // most one checked batch per thread at the end of each colour. (Trimming
 // that last batch to the ceil(rem / nt) slots the block's remaining rem
 // edges need cost 3-6 % on G(n, m) graphs: more code for little saving.)
-template <int K, int B, bool kWrapEach, bool kSgn = false>
+template <int K, int B, bool kWrapEach>
 __device__ __forceinline__ void general_colours_x2(const InstView &a, float *xs, float alpha)
 {
     static_assert(K == 1 || K == 2 || K == 4, "K");
@@ -1421,8 +1398,8 @@ __device__ __forceinline__ void general_colours_x2(const InstView &a, float *xs,
         const int e1 = __ldg(a.off + c + 1);
         int e0 = __ldg(a.off + c) + threadIdx.x;
         for (; e0 + (B - 1) * nt < e1; e0 += B * nt)
-            edge_batch_x2<K, B, kWrapEach, false, false, kSgn>(a, xb, alpha, e0, e1, nt);
-        if (e0 < e1) edge_batch_x2<K, B, kWrapEach, true, false, kSgn>(a, xb, alpha, e0, e1, nt);
+            edge_batch_x2<K, B, kWrapEach, false>(a, xb, alpha, e0, e1, nt);
+        if (e0 < e1) edge_batch_x2<K, B, kWrapEach, true>(a, xb, alpha, e0, e1, nt);
         __syncthreads();
     }
 }
@@ -1697,9 +1674,9 @@ __device__ __forceinline__ void block_pass_odd_h2(H *xs, const uint8_t *wnib, fl
 // per thread, each slot's NW words widened to f32x2 pairs (two replicas a
 // pair), eq. (6) as in the binary32 sweep, and every updated phase wrapped
 // and rounded to the storage type when stored -- after every update, as
-// the oracle's per-update rounding for edge lists has it. kTail and kSgn as
-// in edge_batch_x2.
-template <typename H, int NW, int B, bool kTail, bool kSgn>
+// the oracle's per-update rounding for edge lists has it. kTail as in
+// edge_batch_x2.
+template <typename H, int NW, int B, bool kTail>
 __device__ __forceinline__ void edge_batch_h2(const InstView &a, uint32_t xb, float alpha, int e0, int e1, int nt)
 {
     constexpr uint32_t E = NW * 4;  // bytes per slot
@@ -1711,21 +1688,12 @@ __device__ __forceinline__ void edge_batch_h2(const InstView &a, uint32_t xb, fl
         uint32_t rec = 0;
         int w = 0;
         if (!kTail || e < e1) {
-            if constexpr (kSgn) {
-                rec = load_rec_sgn(a, e);
-            } else {
-                rec = load_rec(a, e);
-                w = __ldg(a.w + e);
-            }
+            rec = load_rec(a, e);
+            w = __ldg(a.w + e);
         }
         aj[u] = xb + (rec >> 16) * E;
-        if constexpr (kSgn) {
-            ai[u] = xb + (rec & 0xFFFEu) * (E / 2);
-            aw[u] = __uint_as_float(flip_if_odd(__float_as_uint(alpha), rec));
-        } else {
-            ai[u] = xb + (rec & 0xFFFFu) * E;
-            aw[u] = alpha * weight_f((int8_t)w);
-        }
+        ai[u] = xb + (rec & 0xFFFFu) * E;
+        aw[u] = alpha * weight_f((int8_t)w);
     }
     f32x2 xi[B][NW], xj[B][NW];
 #pragma unroll
@@ -1754,7 +1722,7 @@ __device__ __forceinline__ void edge_batch_h2(const InstView &a, uint32_t xb, fl
 
 // The colours of one sweep of a 16-bit edge-list tile: whole batches
 // without bounds checks, then at most one checked batch per thread.
-template <typename H, int K, bool kSgn>
+template <typename H, int K>
 __device__ __forceinline__ void general_colours_h2(const InstView &a, H *xs, float alpha)
 {
     constexpr int NW = K / 2, B = K == 8 ? 2 : 3;
@@ -1763,8 +1731,8 @@ __device__ __forceinline__ void general_colours_h2(const InstView &a, H *xs, flo
     for (int c = 0; c < a.C; ++c) {
         const int e1 = __ldg(a.off + c + 1);
         int e0 = __ldg(a.off + c) + threadIdx.x;
-        for (; e0 + (B - 1) * nt < e1; e0 += B * nt) edge_batch_h2<H, NW, B, false, kSgn>(a, xb, alpha, e0, e1, nt);
-        if (e0 < e1) edge_batch_h2<H, NW, B, true, kSgn>(a, xb, alpha, e0, e1, nt);
+        for (; e0 + (B - 1) * nt < e1; e0 += B * nt) edge_batch_h2<H, NW, B, false>(a, xb, alpha, e0, e1, nt);
+        if (e0 < e1) edge_batch_h2<H, NW, B, true>(a, xb, alpha, e0, e1, nt);
         __syncthreads();
     }
 }
@@ -1875,9 +1843,8 @@ __device__ __forceinline__ void sts_w(uint32_t a, const uint32_t (&x)[NW])
 
 // One batch of B edges per thread of the edge-list sweep on packed words
 // (edges e0, e0 + nt, ...); kTail: the batch may run past the end e1 of its
-// colour (its loads and stores skipped there); kSgn: the records of a.ijs,
-// whose bit 0 is the sign of a +-1 weight (no weight load).
-template <int NW, int B, bool kTail, bool kSgn>
+// colour (its loads and stores skipped there).
+template <int NW, int B, bool kTail>
 __device__ __forceinline__ void edge_batch_qw(const InstView &a, uint32_t xb, uint32_t aq, int e0, int e1, int nt)
 {
     constexpr uint32_t E = NW * 4;  // bytes per slot
@@ -1888,21 +1855,12 @@ __device__ __forceinline__ void edge_batch_qw(const InstView &a, uint32_t xb, ui
         uint32_t rec = 0u;
         int32_t w = 0;
         if (!kTail || e < e1) {
-            if constexpr (kSgn) {
-                rec = load_rec_sgn(a, e);
-            } else {
-                rec = load_rec(a, e);
-                w = (int32_t)__ldg(a.w + e);
-            }
+            rec = load_rec(a, e);
+            w = (int32_t)__ldg(a.w + e);
         }
         aj[u] = xb + (rec >> 16) * E;
-        if constexpr (kSgn) {
-            ai[u] = xb + (rec & 0xFFFEu) * (E / 2);
-            pw[u] = (rec & 1u) ? 0u - aq : aq;
-        } else {
-            ai[u] = xb + (rec & 0xFFFFu) * E;
-            pw[u] = (uint32_t)((int32_t)aq * w);
-        }
+        ai[u] = xb + (rec & 0xFFFFu) * E;
+        pw[u] = (uint32_t)((int32_t)aq * w);
     }
     uint32_t xi[B][NW], xj[B][NW];
 #pragma unroll
@@ -1938,13 +1896,8 @@ __device__ __forceinline__ void general_colour_qw(const InstView &a, uint16_t *x
     const uint32_t xb = (uint32_t)__cvta_generic_to_shared(xs);
     const int e1 = __ldg(a.off + c + 1);
     int e0 = __ldg(a.off + c) + threadIdx.x;
-    if (a.ijs) {
-        for (; e0 + (B - 1) * nt < e1; e0 += B * nt) edge_batch_qw<NW, B, false, true>(a, xb, aq, e0, e1, nt);
-        if (e0 < e1) edge_batch_qw<NW, B, true, true>(a, xb, aq, e0, e1, nt);
-    } else {
-        for (; e0 + (B - 1) * nt < e1; e0 += B * nt) edge_batch_qw<NW, B, false, false>(a, xb, aq, e0, e1, nt);
-        if (e0 < e1) edge_batch_qw<NW, B, true, false>(a, xb, aq, e0, e1, nt);
-    }
+    for (; e0 + (B - 1) * nt < e1; e0 += B * nt) edge_batch_qw<NW, B, false>(a, xb, aq, e0, e1, nt);
+    if (e0 < e1) edge_batch_qw<NW, B, true>(a, xb, aq, e0, e1, nt);
 }
 
 // The lattice passes of the fixed-point sweep on packed words (the 2x2
@@ -2333,15 +2286,12 @@ __device__ __forceinline__ void run_segment_fp(const InstView &v, const Segment 
                             general_colours_x2s<K, kB, false>(v, xf, at.x, stage, first, last, stage_cur);
                     } else if (v.wrap_p == 0) {
                         general_colours_x2<K, kB, true>(v, xf, at.x);
-                    } else if (v.ijs) {
-                        general_colours_x2<K, kB, false, true>(v, xf, at.x);
                     } else {
                         general_colours_x2<K, kB, false>(v, xf, at.x);
                     }
                 } else {
                     // 16-bit storage: f32x2 lanes over the replica pairs of a word
-                    if (v.ijs) general_colours_h2<Store, K, true>(v, t.xs, at.x);
-                    else general_colours_h2<Store, K, false>(v, t.xs, at.x);
+                    general_colours_h2<Store, K>(v, t.xs, at.x);
                 }
                 if (v.hv) {
                     field_pass<Store, K>(v, t.xs, at.x);

@@ -101,7 +101,6 @@ struct cosm_handle {
     int32_t C = 0;
     DevBuf<uint32_t> d_ij;
     DevBuf<int8_t> d_w;
-    DevBuf<uint32_t> d_ijs;         // +-1 weights on <= 2^15 slots: records with the sign in bit 31
     std::vector<uint32_t> h_ij;     // colour-major records and weights on the host
     std::vector<int8_t> h_wv;
     std::vector<std::unique_ptr<cosm::RecordTable>> tables;

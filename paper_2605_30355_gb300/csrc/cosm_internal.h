@@ -38,10 +38,6 @@ struct InstView {
     const int32_t *off;   // device: colour offsets into ij / w (C + 1)
     const uint32_t *ij;   // edge records: slot(src) | slot(dst) << 16, colour-major
     const int8_t *w;      // Max-Cut weights, colour-major
-    // the same records for +-1 weights on at most 2^15 slots with the weight
-    // in bit 0 ([w = -1] | slot(src) << 1 | slot(dst) << 16), so the
-    // binary32 edge-list sweep loads one word per edge; nullptr otherwise
-    const uint32_t *ijs;
     // the same edges as a record table for this launch's tile width and thread
     // count (cosm_edges.h): n_colours non-empty colours
     const uint32_t *rec;

@@ -133,7 +133,7 @@ extern "C" void cosm_destroy(cosm_handle *h)
 {
     if (!h) return;
     if (h->stream || h->have_state) cudaStreamSynchronize(h->stream);
-    h->d_ij.release(); h->d_w.release(); h->d_ijs.release(); h->d_orig.release(); h->d_slot.release(); h->d_off.release(); h->d_state.release();
+    h->d_ij.release(); h->d_w.release(); h->d_orig.release(); h->d_slot.release(); h->d_off.release(); h->d_state.release();
     h->d_cut.release(); h->d_bestp.release(); h->d_alpha.release(); h->d_segs.release();
     h->d_segoff.release(); h->d_ready.release(); h->d_err.release(); h->d_best.release();
     h->d_spins.release();
@@ -463,22 +463,6 @@ extern "C" int cosm_create(const cosm_graph_desc *gd, const cosm_params *p, cosm
             return fail(COSM_ERR_CUDA, "copying the graph to the device failed");
         }
     }
-    // +-1 weights on at most 2^15 slots: the weight folded into the record
-    bool unit = g.n <= (1 << 15);
-    for (int64_t k = 0; unit && k < g.m; ++k) unit = wv[(size_t)k] == 1 || wv[(size_t)k] == -1;
-    if (unit) {
-        std::vector<uint32_t> ijs(m_pad, 0u);
-        for (int64_t k = 0; k < g.m; ++k)
-            ijs[(size_t)k] = ((ij[(size_t)k] & 0xFFFFu) << 1) | (ij[(size_t)k] & 0xFFFF0000u) | (wv[(size_t)k] < 0 ? 1u : 0u);
-        if ((rc = h->d_ijs.ensure(m_pad))) {
-            cosm_destroy(h);
-            return rc;
-        }
-        if (cudaMemcpy(h->d_ijs.p, ijs.data(), ijs.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess) {
-            cosm_destroy(h);
-            return fail(COSM_ERR_CUDA, "copying the graph to the device failed");
-        }
-    }
     if (h->fields) {
         std::vector<int32_t> hs((size_t)g.n);
         for (int32_t v = 0; v < g.n; ++v) hs[(size_t)h->slot_of[(size_t)v]] = gd->h[v];
@@ -728,7 +712,7 @@ static int record_format(const cosm_handle *h, int K)
     const int E = K * (p.storage == COSM_F32 ? 4 : 2);
     const bool each = p.storage == COSM_F32 && wrap_period(p.alpha0_deg, p.dwt_ratio, p.dwt_period, p.flags, h->mode,
                                                            p.storage, h->wbound) == 0;
-    if (h->d_ijs.p && !each) return EDGES_SIGN;
+    if (h->wmax == 1 && h->g.n <= (1 << 15) && !each) return EDGES_SIGN;
     const int more = each ? EDGES_EACH : 0;
     // one word (half the record traffic of a weighted graph) where it holds
     if (E >= 8 && h->g.n <= (1 << 14) && h->wmax <= (E == 8 ? 3 : 7)) return EDGES_PACK | more;
@@ -1150,8 +1134,6 @@ InstView cosm::inst_view(cosm_handle *h)
     v.off = h->d_off.p;
     v.ij = h->d_ij.p;
     v.w = h->d_w.p;
-    // test hook: COSM_SPLIT_W keeps the split records and weights
-    v.ijs = std::getenv("COSM_SPLIT_W") ? nullptr : h->d_ijs.p;
     v.orig_of = h->d_orig.p;
     v.slot_of = h->d_slot.p;
     v.wnib = h->d_wnib.p;
