@@ -560,17 +560,17 @@ def run_ours(args):
 
 # ncu records of the sweep kernel's memory traffic on the bench's workloads,
 # each taken at the kernel source whose hash it names (the first 12 hex
-# digits of the SHA-256 of cosm_kernels.cu): reported only while that source
+# digits of the SHA-256 of the device code's files): reported only while that source
 # is unchanged, else null. Keys: (workload, storage). Values: shared-memory
 # bytes per edge-replica update (shared wavefronts x 128 B / updates, from a
 # small capture of the same kernel and layout), and DRAM bytes (read +
 # write) of one full-size launch with its (replicas, sweeps) -- DRAM traffic
 # follows the state, not the sweeps, so it is not scaled from a small case.
 NCU_TRAFFIC = {
-    ("torus20k", "f32"): (8.60, (83.37e6, 1024, 100_000), "1bcbe8654a3b"),
-    ("torus20k", "f16"): (4.43, None, "1bcbe8654a3b"),
-    ("torus20k", "q16"): (4.39, None, "1bcbe8654a3b"),
-    ("reg3_20k", "f32"): (22.5, None, "1bcbe8654a3b"),
+    ("torus20k", "f32"): (3.23, None, "a44eb127ec7d"),
+    ("torus20k", "f16"): (4.39, None, "a44eb127ec7d"),
+    ("torus20k", "q16"): (1.66, None, "a44eb127ec7d"),
+    ("reg3_20k", "f32"): (21.7, None, "a44eb127ec7d"),
 }
 
 # Algorithmic cost of one edge-replica update of eq. (6): FP32 operations
@@ -580,10 +580,16 @@ ALU_OPS_PER_UPDATE = 6
 
 
 def kernel_source_hash():
+    """Of everything the device code is compiled from."""
+    import glob
     import hashlib
-    path = os.path.join(ROOT, "paper_2605_30355_gb300", "csrc", "cosm_kernels.cu")
-    with open(path, "rb") as f:
-        return hashlib.sha256(f.read()).hexdigest()[:12]
+    csrc = os.path.join(ROOT, "paper_2605_30355_gb300", "csrc")
+    digest = hashlib.sha256()
+    for pattern in ("cosm_*.cuh", "cosm_patch_*.cu", "cosm_edges_*.cu", "cosm_kernels.cu"):
+        for path in sorted(glob.glob(os.path.join(csrc, pattern))):
+            with open(path, "rb") as f:
+                digest.update(f.read())
+    return digest.hexdigest()[:12]
 
 
 _PROBES = {}
