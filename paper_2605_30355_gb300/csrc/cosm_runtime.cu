@@ -129,6 +129,17 @@ extern "C" int cosm_color_torus3d(int32_t L1, int32_t L2, int32_t L3, int64_t m,
 
 // ------------------------------------------------------------------ create
 
+// Waits for the copies made on the legacy stream. cudaMemcpy from pageable
+// memory may return while its transfer is still queued there, and a stream
+// created non-blocking -- a batch's, a server's, a caller's -- does not wait
+// for the legacy stream: whatever is copied this way for a later launch has
+// arrived before the call that copies it returns.
+static int settle()
+{
+    CK(cudaStreamSynchronize(nullptr));
+    return COSM_OK;
+}
+
 extern "C" void cosm_destroy(cosm_handle *h)
 {
     if (!h) return;
@@ -482,7 +493,7 @@ extern "C" int cosm_create(const cosm_graph_desc *gd, const cosm_params *p, cosm
             return fail(COSM_ERR_CUDA, "copying the local fields to the device failed");
         }
     }
-    if ((rc = setup_lattice2d(h, pattern))) {
+    if ((rc = setup_lattice2d(h, pattern)) || (rc = settle())) {
         cosm_destroy(h);
         return rc;
     }
@@ -692,7 +703,7 @@ static int ensure_patch_weights(cosm_handle *h)
     }
     int rc = buf.ensure(wt.size());
     if (rc) return rc;
-    if (cudaMemcpy(buf.p, wt.data(), wt.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess) {
+    if (cudaMemcpy(buf.p, wt.data(), wt.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess || settle()) {
         buf.release();
         return fail(COSM_ERR_CUDA, "copying the patch weights to the device failed");
     }
@@ -923,7 +934,7 @@ static int ensure_records(cosm_handle *h)
     }
     if (cudaMemcpy(t->rec.p, rec.data(), rec.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(t->counts.p, counts.data(), counts.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(t->starts.p, starts.data(), (size_t)W * 4, cudaMemcpyHostToDevice) != cudaSuccess) {
+        cudaMemcpy(t->starts.p, starts.data(), (size_t)W * 4, cudaMemcpyHostToDevice) != cudaSuccess || settle()) {
         t->release();
         return fail(COSM_ERR_CUDA, "copying the record table to the device failed");
     }
@@ -1571,8 +1582,7 @@ static int state_rows(cosm_handle *h, int kind, void *rows)
             return fail(COSM_ERR_CUDA, std::string("state launch: ") + cudaGetErrorString(cudaGetLastError()));
         if (kind >= 0) CK(cudaMemcpy(part, h->d_stage.p, (size_t)(r1 - r0) * row, cudaMemcpyDefault));
     }
-    CK(cudaStreamSynchronize(nullptr));
-    return COSM_OK;
+    return settle();
 }
 
 extern "C" int cosm_get_state(cosm_handle *h, double *phases)
@@ -1624,6 +1634,7 @@ extern "C" int cosm_set_state(cosm_handle *h, const double *phases, int32_t repl
         }
     }
     CK(cudaMemcpy(h->d_state.p, raw.data(), raw.size(), cudaMemcpyHostToDevice));
+    if ((rc = settle())) return rc;
     h->have_state = true;
     h->sweep_idx = 0;
     h->have_result = false;
@@ -1714,7 +1725,7 @@ extern "C" int cosm_step(cosm_handle *h, int64_t sweep, float alpha, void *strea
                                        (float)std::floor(h->prm.dwt_ratio * (double)alpha * 65536.0 + 0.5))
                          : make_float2(alpha, (float)(h->prm.dwt_ratio * (double)alpha));
     if (h->stream) CK(cudaStreamSynchronize(h->stream));
-    if (cudaMemcpy(tab.p, &v, sizeof(v), cudaMemcpyHostToDevice) != cudaSuccess) {
+    if (cudaMemcpyAsync(tab.p, &v, sizeof(v), cudaMemcpyHostToDevice, st) != cudaSuccess) {
         tab.release();
         return fail(COSM_ERR_CUDA, "alpha upload failed");
     }

@@ -1,0 +1,105 @@
+"""The host runtime without a GPU: its own sources linked with a stand-in for
+the CUDA runtime and the kernels (fake_device.cpp), which checks every launch
+for copies still on their way, for tables of another layout and for states
+read in another layout than they were written in."""
+import ctypes as C
+import importlib.util
+import os
+import subprocess
+import sys
+
+import numpy as np
+import pytest
+
+import instances
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+PKG = os.path.join(ROOT, "paper_2605_30355_gb300")
+STREAM = 0x50  # a caller's stream
+
+
+def build_fake(out):
+    sys.path.insert(0, ROOT)
+    from paper_2605_30355_gb300 import build
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build.nvcc()))), "include")
+    src = [os.path.join(ROOT, "tests", "fake_device.cpp")] + \
+        [os.path.join(PKG, "csrc", f) for f in ("cosm_runtime.cu", "cosm_server.cu", "cosm_graph.cpp")]
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-w", "-I", os.path.join(PKG, "csrc"), "-I",
+                           os.path.join(ROOT, "include"), "-I", cuda, "-x", "c++"] + src +
+                          ["-o", out, "-static-libstdc++", "-static-libgcc", "-Wl,-Bsymbolic", "-ldl", "-lpthread"])
+    return out
+
+
+def load_fake(path):
+    """A second copy of the package, bound to the library at `path`."""
+    spec = importlib.util.spec_from_file_location("cosm_on_fake", os.path.join(PKG, "__init__.py"),
+                                                  submodule_search_locations=[PKG])
+    cosm = importlib.util.module_from_spec(spec)
+    sys.modules["cosm_on_fake"] = cosm
+    spec.loader.exec_module(cosm)
+    cosm.LIB_PATH = path
+    lib = cosm.lib()
+    lib.fake_message.restype = C.c_char_p
+    lib.fake_live_bytes.restype = C.c_int64
+    lib.fake_fail_malloc.argtypes = [C.c_int64]
+    return cosm
+
+
+@pytest.fixture(scope="session")
+def fake_path(tmp_path_factory):
+    return build_fake(str(tmp_path_factory.mktemp("fake") / "libcosm_host.so"))
+
+
+@pytest.fixture
+def cosm(fake_path):
+    cosm = load_fake(fake_path)
+    report(cosm)
+    return cosm
+
+
+def report(cosm):
+    """What the launches since the last report were, and what was wrong with them."""
+    out = (C.c_int64 * 8)()
+    msg = cosm.lib().fake_message().decode()
+    cosm.lib().fake_report(out)
+    return dict(zip(("unordered", "bad", "launches", "threads", "K", "shape", "ragged", "format"), out), message=msg)
+
+
+def sound(cosm):
+    r = report(cosm)
+    assert r["bad"] == 0 and r["unordered"] == 0, r
+    return r
+
+
+GRAPHS = {"edges": lambda: instances.sparse_gnm(900, 2400, 1), "lattice": lambda: instances.torus2d(40, 60, 1)}
+
+
+@pytest.mark.parametrize("graph", GRAPHS)
+def test_uploads_arrive_before_launches_on_other_streams(cosm, graph):
+    # a copy from pageable memory may still be queued on the legacy stream when
+    # cudaMemcpy returns; streams created non-blocking do not wait for it
+    inst = GRAPHS[graph]()
+    s = cosm.Solver.from_instance(inst)
+    for replicas in (4, 4096, 4):  # a new layout each time
+        s.run(20, replicas, 1, stream=STREAM)
+        sound(cosm)
+    s.set_state(np.zeros((4, inst.n)))
+    s.step(1, 0.01, stream=STREAM)
+    s.import_state(s.export_state()[0], 4, 1, 5)
+    s.run_range(20, 6, 20, 4, 1, stream=STREAM)
+    s.readout(stream=STREAM)
+    sound(cosm)
+
+
+def test_batch_and_server_uploads_arrive_before_their_launches(cosm):
+    insts = [g() for g in GRAPHS.values()] * 3
+    b = cosm.Batch(insts)
+    b.run(20, 4, 1)
+    sound(cosm)
+    b.run(20, 4096, 1)  # other layouts
+    sound(cosm)
+    srv = cosm.Server(chunk_sweeps=7)
+    for rid in [srv.submit(inst, 20, 4, 1, 10 ** 9) for inst in insts]:
+        assert srv.wait(rid, 60)["status"] == cosm.EXHAUSTED
+    srv.close()
+    sound(cosm)
