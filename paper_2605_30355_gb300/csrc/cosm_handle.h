@@ -82,9 +82,24 @@ struct RecordTable {
     }
 };
 
+// How a handle's replicas are laid out in tiles: the kernel and tables that
+// its launches take, and the layout its state is stored in.
+struct TileLayout {
+    int K = 0, threads = 0, occupancy = 0;
+    int shape = -1;            // patch shape of the register kernels (-1: phases in shared memory)
+    bool ragged = false;       // the shape does not divide the lattice
+    int pgr = 0, pgc = 0, pfr = 0, pfc = 0;  // patch grid and its whole rows / columns of patches
+    int format = -1;           // record-table format (-1: none)
+    const RecordTable *table = nullptr;      // its table
+    bool block_pairs = false;  // binary32 lattice tiles of two replicas: two 2x2 blocks per thread (even pass)
+    bool staged = false;       // binary32 edge lists: colour records staged in shared memory
+    size_t smem = 0;
+    int64_t tile_stride = 0;   // storage elements per tile
+};
+
 }  // namespace cosm
 
-struct cosm_handle {
+struct cosm_handle : cosm::TileLayout {
     using Graph = cosm::Graph;
     template <typename T> using DevBuf = cosm::DevBuf<T>;
     Graph g;                        // host copy, original vertex ids
@@ -104,8 +119,6 @@ struct cosm_handle {
     std::vector<uint32_t> h_ij;     // colour-major records and weights on the host
     std::vector<int8_t> h_wv;
     std::vector<std::unique_ptr<cosm::RecordTable>> tables;
-    const cosm::RecordTable *table = nullptr;  // the current layout's
-    int format = -1;                // record-table format of the current layout (-1: none)
     DevBuf<int32_t> d_orig;
     DevBuf<uint16_t> d_slot;        // original id -> slot (lattices)
     DevBuf<int32_t> d_off;          // colour offsets
@@ -151,14 +164,7 @@ struct cosm_handle {
     bool segs_uploaded = false;
     // state of the last launch
     int replicas = 0;
-    int K = 0, threads = 0, occupancy = 0, grid = 0;
-    int shape = -1;            // patch shape of the register kernels (-1: phases in shared memory)
-    bool ragged = false;       // the shape does not divide the lattice
-    int pgr = 0, pgc = 0, pfr = 0, pfc = 0;  // patch grid and its whole rows / columns of patches
-    bool block_pairs = false;  // binary32 lattice tiles of two replicas: two 2x2 blocks per thread (even pass)
-    bool staged = false;       // binary32 edge lists: colour records staged in shared memory
-    size_t smem = 0;
-    int64_t tile_stride = 0;  // storage elements per tile
+    int grid = 0;
     uint64_t seed = 0;
     int64_t sweep_idx = 0;          // sweeps of the current trial applied to the state
     int64_t target = INT64_MIN;     // success threshold of the last run's cuts

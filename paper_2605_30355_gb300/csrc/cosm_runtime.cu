@@ -922,6 +922,7 @@ static int ensure_records(cosm_handle *h)
         std::copy_n(rec.begin() + starts[(size_t)w],
                     std::min(kRowsAhead * 32 * RW, at[(size_t)w] - starts[(size_t)w]), rec.begin() + at[(size_t)w]);
     std::unique_ptr<RecordTable> t(new RecordTable());
+    h->tables.reserve(h->tables.size() + 1);
     t->K = h->K;
     t->threads = h->threads;
     t->format = h->format;
@@ -1363,6 +1364,26 @@ int cosm::launch_finalize(cosm_handle *h, cudaStream_t st)
     return COSM_OK;
 }
 
+// The layout, tables and buffers of `replicas` replicas. Where no layout fits
+// or its tables cannot be built the handle keeps the layout it had, with the
+// state and results that are stored in it; a new layout ends them.
+static int prepare_replicas(cosm_handle *h, int32_t replicas)
+{
+    const auto forget = [h] { h->have_state = h->have_result = h->have_trace = h->bits_valid = false; };
+    int rc;
+    if (!h->K || replicas != h->replicas) {
+        const TileLayout before = *h;
+        if ((rc = choose_layout(h, replicas)) || (rc = ensure_tables(h))) {
+            static_cast<TileLayout &>(*h) = before;
+            return rc;
+        }
+        h->replicas = replicas;
+        forget();
+    }
+    if ((rc = ensure_run_buffers(h, replicas))) forget();
+    return rc;
+}
+
 // Sweeps s0..s1 of an S-sweep trial of every replica (cosm_run: 1..S).
 static int run_range(cosm_handle *h, int64_t sweeps, int64_t s0, int64_t s1, int32_t replicas, uint64_t seed,
                      int64_t target_cut, cudaStream_t st)
@@ -1381,13 +1402,10 @@ static int run_range(cosm_handle *h, int64_t sweeps, int64_t s0, int64_t s1, int
         if (replicas != h->replicas || seed != h->seed)
             return fail(COSM_ERR_INVALID_ARG, "a continued trial keeps its replica count and seed");
         if (h->stream && h->stream != st) CK(cudaStreamSynchronize(h->stream));
-    } else if (!h->K || replicas != h->replicas) {
-        if ((rc = choose_layout(h, replicas)) || (rc = ensure_tables(h))) return rc;
     }
-    h->replicas = replicas;
+    if ((rc = prepare_replicas(h, replicas))) return rc;
     h->seed = seed;
     h->target = target_cut;
-    if ((rc = ensure_run_buffers(h, replicas))) return rc;
     if ((rc = upload_alpha(h, sweeps, st))) return rc;
     const int64_t tiles = (replicas + h->K - 1) / h->K;
     int64_t cap = (int64_t)h->occupancy * h->num_sms;
@@ -1600,22 +1618,19 @@ extern "C" int cosm_set_state(cosm_handle *h, const double *phases, int32_t repl
     if (replicas < 1 || replicas >= (1 << 24)) return fail(COSM_ERR_INVALID_ARG, "bad replica count");
     int rc;
     if (h->stream) CK(cudaStreamSynchronize(h->stream));
-    if (!h->K || replicas != h->replicas) {
-        if ((rc = choose_layout(h, replicas)) || (rc = ensure_tables(h))) return rc;
-    }
-    h->replicas = replicas;
-    h->seed = seed;
-    if ((rc = ensure_run_buffers(h, replicas))) return rc;
     std::vector<double> in((size_t)replicas * h->g.n);
     CK(cudaMemcpy(in.data(), phases, in.size() * 8, cudaMemcpyDefault));
+    for (double x : in)
+        if (!(x >= 0.0 && x < 1.0)) return fail(COSM_ERR_INVALID_ARG, "phases must be in [0, 1)");
+    if ((rc = prepare_replicas(h, replicas))) return rc;
+    h->seed = seed;
     const int64_t tiles = (replicas + h->K - 1) / h->K;
     const size_t esz = h->prm.storage == COSM_F32 ? 4 : 2;
     std::vector<unsigned char> raw((size_t)tiles * (size_t)h->tile_stride * esz, 0);
     for (int32_t r = 0; r < replicas; ++r) {
         const size_t base = (size_t)(r / h->K) * (size_t)h->tile_stride;
         for (int32_t v = 0; v < h->g.n; ++v) {
-            double x = in[(size_t)r * h->g.n + v] + 0.0;  // -0 becomes +0
-            if (!(x >= 0.0 && x < 1.0)) return fail(COSM_ERR_INVALID_ARG, "phases must be in [0, 1)");
+            const double x = in[(size_t)r * h->g.n + v] + 0.0;  // -0 becomes +0
             const double g = x >= 0.5 ? x - 1.0 : x;
             const size_t idx = base + (size_t)h->slot_of[(size_t)v] * h->K + (size_t)(r % h->K);
             if (esz == 4) {
@@ -1664,12 +1679,8 @@ extern "C" int cosm_import_state(cosm_handle *h, const void *phases, int32_t sto
     if (sweep_idx < 0 || sweep_idx >= ((int64_t)1 << 31)) return fail(COSM_ERR_INVALID_ARG, "bad sweep index");
     int rc;
     if (h->stream) CK(cudaStreamSynchronize(h->stream));
-    if (!h->K || replicas != h->replicas) {
-        if ((rc = choose_layout(h, replicas)) || (rc = ensure_tables(h))) return rc;
-    }
-    h->replicas = replicas;
+    if ((rc = prepare_replicas(h, replicas))) return rc;
     h->seed = seed;
-    if ((rc = ensure_run_buffers(h, replicas))) return rc;
     if ((rc = state_rows(h, -1, const_cast<void *>(phases)))) return rc;
     h->have_state = true;
     h->sweep_idx = sweep_idx;
@@ -2002,13 +2013,9 @@ static int batch_layout(cosm_batch *b, const int64_t *sweeps, const int32_t *rep
     std::vector<InstView> views((size_t)n);
     std::vector<BatchFinal> fins((size_t)n);
     double total = 0.0;  // edge updates of the run
-    for (int i = 0; i < n; ++i)
-        if (sweeps[i] > 0 && replicas[i] > 0)
-            total += (double)b->hs[(size_t)i]->g.m * (double)replicas[i] * (double)sweeps[i];
+    for (int i = 0; i < n; ++i) total += (double)b->hs[(size_t)i]->g.m * (double)replicas[i] * (double)sweeps[i];
     for (int i = 0; i < n; ++i) {
         cosm_handle *h = b->hs[(size_t)i];
-        if (sweeps[i] < 1 || sweeps[i] >= ((int64_t)1 << 31) || replicas[i] < 1 || replicas[i] >= (1 << 24))
-            return fail(COSM_ERR_INVALID_ARG, "instance " + std::to_string(i) + ": bad sweeps or replicas");
         int rc;
         const double fill = 0.6 * total / ((double)h->g.m * (double)sweeps[i]);
         if ((rc = batch_instance_layout(b, h, replicas[i], (int32_t)std::max((double)replicas[i],
@@ -2142,6 +2149,9 @@ extern "C" int cosm_batch_run(cosm_batch *b, const int64_t *sweeps, const int32_
 {
     NvtxRange range("cosm_batch_run");
     if (!b || !sweeps || !replicas || !seeds) return fail(COSM_ERR_INVALID_ARG, "NULL argument");
+    for (size_t i = 0; i < b->hs.size(); ++i)
+        if (sweeps[i] < 1 || sweeps[i] >= ((int64_t)1 << 31) || replicas[i] < 1 || replicas[i] >= (1 << 24))
+            return fail(COSM_ERR_INVALID_ARG, "instance " + std::to_string(i) + ": bad sweeps or replicas");
     cudaStream_t user = reinterpret_cast<cudaStream_t>(stream);
     cudaStream_t st = b->own;
     // order the batch after earlier work on the caller's stream
@@ -2151,7 +2161,12 @@ extern "C" int cosm_batch_run(cosm_batch *b, const int64_t *sweeps, const int32_
     CK(cudaStreamWaitEvent(st, e0, 0));
     cudaEventDestroy(e0);
     int rc = batch_layout(b, sweeps, replicas, seeds, st);
-    if (rc) return rc;
+    if (rc) {
+        // some instances have a new layout: the last run's states and results end here
+        for (cosm_handle *h : b->hs) h->have_state = h->have_result = false;
+        b->have_result = false;
+        return rc;
+    }
     std::vector<int64_t> sig;
     sig.push_back((int64_t)(uintptr_t)b->d_insts.p);
     sig.push_back((int64_t)(uintptr_t)b->d_units.p);

@@ -103,3 +103,87 @@ def test_batch_and_server_uploads_arrive_before_their_launches(cosm):
         assert srv.wait(rid, 60)["status"] == cosm.EXHAUSTED
     srv.close()
     sound(cosm)
+
+
+@pytest.mark.parametrize("entry", ["run", "set_state", "import_state"])
+@pytest.mark.parametrize("graph", GRAPHS)
+def test_failed_tables_leave_the_layout_of_the_state(cosm, graph, entry):
+    # a run whose tables do not fit in device memory changes nothing: the
+    # earlier run's state and results stay readable, and its replica count runs
+    # again on its own kernel and table
+    inst = GRAPHS[graph]()
+    s = cosm.Solver.from_instance(inst)
+    s.run(20, 4, 1)
+    first = sound(cosm)
+    lay = s.layout()
+    cosm.lib().fake_fail_malloc(1)
+    many = 4096
+    with pytest.raises(cosm.CosmError) as err:
+        if entry == "run":
+            s.run(20, many, 1)
+        elif entry == "set_state":
+            s.set_state(np.zeros((many, inst.n)))
+        else:
+            s.import_state(np.zeros((many, inst.n), np.float32), many, 1, 0)
+    assert err.value.code == cosm.ERR_NOMEM
+    s.replicas = 4
+    assert s.layout() == lay
+    s.export_state()
+    s.replica_cuts()
+    s.readout()
+    s.run(20, 4, 1)
+    again = sound(cosm)
+    assert [again[k] for k in ("K", "threads", "shape", "format")] == \
+        [first[k] for k in ("K", "threads", "shape", "format")]
+    # with memory there, the larger run takes another layout, which is what
+    # the failure must not leave behind
+    s.run(20, many, 1)
+    other = sound(cosm)
+    assert [other[k] for k in ("K", "threads", "shape")] != [first[k] for k in ("K", "threads", "shape")]
+    s.run(20, 4, 1)
+    sound(cosm)
+
+
+@pytest.mark.parametrize("nth", range(2, 8))
+def test_failed_buffers_end_the_state(cosm, nth):
+    # the state's buffer may be gone or of another layout: no call reads it
+    s = cosm.Solver.from_instance(GRAPHS["edges"]())
+    s.run(20, 4, 1)
+    sound(cosm)
+    cosm.lib().fake_fail_malloc(nth + 2)  # the table's three buffers, then those of the run
+    with pytest.raises(cosm.CosmError) as err:
+        s.run(20, 4096, 1)
+    assert err.value.code == cosm.ERR_NOMEM
+    for call in (s.export_state, s.replica_cuts, s.readout, lambda: s.step(1, 0.01)):
+        with pytest.raises(cosm.CosmError) as err:
+            call()
+        assert err.value.code == cosm.ERR_STATE
+    s.run(20, 4, 1)
+    s.export_state()
+    sound(cosm)
+
+
+def test_failed_batch_run_ends_the_batch_state(cosm):
+    insts = [g() for g in GRAPHS.values()]
+    b = cosm.Batch(insts)
+    b.run([20, 20], [4, 4], [1, 2])
+    for bad in (0, 1 << 24):  # refused arguments change nothing
+        with pytest.raises(cosm.CosmError) as err:
+            b.run([20, 20], [4096, bad], [1, 2])
+        assert err.value.code == cosm.ERR_INVALID_ARG
+    b.replicas = [4, 4]
+    b.get_state(0)
+    sound(cosm)
+    cosm.lib().fake_fail_malloc(1)
+    with pytest.raises(cosm.CosmError) as err:
+        b.run([20, 20], [4096, 4096], [1, 2])
+    assert err.value.code == cosm.ERR_NOMEM
+    b.replicas = [4, 4]
+    for call in (b.get_state, b.best, b.replica_cuts):
+        with pytest.raises(cosm.CosmError) as err:
+            call(0)
+        assert err.value.code == cosm.ERR_STATE
+    b.run([20, 20], [4096, 4096], [1, 2])
+    b.get_state(1)
+    b.close()
+    assert report(cosm)["bad"] == 0
