@@ -5,9 +5,13 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstdint>
 #include <memory>
+#include <new>
 #include <string>
+#include <system_error>
+#include <thread>
 #include <vector>
 
 #include "../../include/cosm.h"
@@ -196,5 +200,32 @@ int upload_alpha(cosm_handle *h, int64_t S, cudaStream_t st);
 int launch_finalize(cosm_handle *h, cudaStream_t st);
 int launch_opt_readout(cosm_handle *h, bool keep_better, cudaStream_t st);
 int single_only(const cosm_graph_desc *g, const cosm_params *p);
+
+// Runs work(i) for i < count on the calling thread and at most 15 more, each
+// with `device` current. Where no more threads can be created the ones there do
+// the work. Returns how many took part.
+template <typename Work>
+int side_by_side(size_t count, int device, const Work &work)
+{
+    std::atomic<size_t> next{0};
+    const auto loop = [&] {
+        for (size_t i; (i = next++) < count;) work(i);
+    };
+    std::vector<std::thread> pool;
+    const size_t most = std::min<size_t>(count, std::max(1u, std::min(16u, std::thread::hardware_concurrency())));
+    try {
+        pool.reserve(most);
+        while (pool.size() + 1 < most)
+            pool.emplace_back([&loop, device] {
+                cudaSetDevice(device);
+                loop();
+            });
+    } catch (const std::system_error &) {
+    } catch (const std::bad_alloc &) {
+    }
+    loop();
+    for (auto &t : pool) t.join();
+    return (int)pool.size() + 1;
+}
 
 }  // namespace cosm

@@ -9,7 +9,6 @@
 #include <cstdlib>
 #include <cstring>
 #include <string>
-#include <thread>
 #include <vector>
 
 #include "../../include/cosm.h"
@@ -1886,26 +1885,14 @@ extern "C" int cosm_batch_create(int32_t count, const cosm_graph_desc *graphs, c
     b->hs.assign((size_t)count, nullptr);
     std::vector<int> rcs((size_t)count, COSM_OK);
     std::vector<std::string> msgs((size_t)count);
-    const int workers = (int)std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
-    auto work = [&](int t) {
-        cudaSetDevice(dev);
-        for (int32_t i = t; i < count; i += workers) {
-            const cosm_params *pi = shared_params ? &params[0] : &params[i];
-            const int rc = cosm_create(&graphs[i], pi, &b->hs[(size_t)i]);
-            if (rc) {
-                rcs[(size_t)i] = rc;
-                msgs[(size_t)i] = g_err;
-            }
-        }
+    const auto work = [&](size_t i) {
+        const cosm_params *pi = shared_params ? &params[0] : &params[i];
+        if ((rcs[i] = cosm_create(&graphs[i], pi, &b->hs[i]))) msgs[i] = g_err;
     };
-    if (workers == 1 || count < 4) {
-        work(0);
-        for (int t = 1; t < workers; ++t) work(t);
-    } else {
-        std::vector<std::thread> pool;
-        for (int t = 0; t < workers; ++t) pool.emplace_back(work, t);
-        for (auto &th : pool) th.join();
-    }
+    if (count < 4)
+        for (size_t i = 0; i < (size_t)count; ++i) work(i);
+    else
+        side_by_side((size_t)count, dev, work);
     for (int32_t i = 0; i < count; ++i) {
         if (rcs[(size_t)i]) {
             std::string msg = "instance " + std::to_string(i) + ": " + msgs[(size_t)i];
@@ -1958,21 +1945,6 @@ static int batch_instance_layout(cosm_batch *b, cosm_handle *h, int32_t replicas
     return COSM_OK;
 }
 
-// Runs work(t) for t = 0 .. workers - 1 on host threads, each with the
-// caller's device current.
-template <typename Work>
-static void on_workers(int workers, int dev, const Work &work)
-{
-    std::vector<std::thread> pool;
-    for (int t = 1; t < workers; ++t)
-        pool.emplace_back([&work, dev, t] {
-            cudaSetDevice(dev);
-            work(t);
-        });
-    work(0);
-    for (auto &th : pool) th.join();
-}
-
 // The device tables of every instance's layout. Missing ones (a first run, or
 // another layout) are built by host threads side by side.
 static int batch_tables(cosm_batch *b)
@@ -1994,12 +1966,10 @@ static int batch_tables(cosm_batch *b)
     if (todo.empty()) return COSM_OK;
     int dev = 0;
     CK(cudaGetDevice(&dev));
-    const int workers = (int)std::min<size_t>(todo.size(), std::max(1u, std::min(16u, std::thread::hardware_concurrency())));
     std::vector<int> rcs(todo.size(), COSM_OK);
     std::vector<std::string> msgs(todo.size());
-    on_workers(workers, dev, [&](int t) {
-        for (size_t i = (size_t)t; i < todo.size(); i += (size_t)workers)
-            if ((rcs[i] = ensure_tables(todo[i]))) msgs[i] = g_err;
+    side_by_side(todo.size(), dev, [&](size_t i) {
+        if ((rcs[i] = ensure_tables(todo[i]))) msgs[i] = g_err;
     });
     for (size_t i = 0; i < todo.size(); ++i)
         if (rcs[i]) return fail(rcs[i], msgs[i]);

@@ -13,7 +13,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <atomic>
 #include <chrono>
 #include <climits>
 #include <condition_variable>
@@ -21,7 +20,6 @@
 #include <deque>
 #include <mutex>
 #include <string>
-#include <system_error>
 #include <thread>
 #include <unordered_map>
 #include <vector>
@@ -138,23 +136,7 @@ static int admit(cosm_server *s, Request *r)
 static std::vector<int> admit_all(cosm_server *s, const std::vector<Request *> &fresh)
 {
     std::vector<int> rcs(fresh.size(), COSM_OK);
-    std::atomic<size_t> next{0};
-    auto work = [&] {
-        for (size_t i; (i = next++) < fresh.size();) rcs[i] = admit(s, fresh[i]);
-    };
-    const size_t most = std::min<size_t>(fresh.size(), std::max(1u, std::min(16u, std::thread::hardware_concurrency())));
-    std::vector<std::thread> pool;
-    pool.reserve(most);
-    try {
-        while (pool.size() + 1 < most)
-            pool.emplace_back([&] {
-                cudaSetDevice(s->device);
-                work();
-            });
-    } catch (const std::system_error &) {  // no more threads: the ones there do the work
-    }
-    work();
-    for (auto &t : pool) t.join();
+    const int threads = side_by_side(fresh.size(), s->device, [&](size_t i) { rcs[i] = admit(s, fresh[i]); });
     // device memory that ran out goes to the requests in arrival order: all
     // from the first one that had none are admitted again, one by one
     size_t i = 0;
@@ -163,7 +145,7 @@ static std::vector<int> admit_all(cosm_server *s, const std::vector<Request *> &
         if (r->h) cosm_destroy(r->h);
         r->h = nullptr;
     };
-    if (pool.empty()) i = rcs.size();  // they were
+    if (threads == 1) i = rcs.size();  // they were
     for (size_t k = i; k < rcs.size(); ++k) drop(fresh[k]);
     for (; i < rcs.size(); ++i)
         if ((rcs[i] = admit(s, fresh[i]))) drop(fresh[i]);
@@ -419,7 +401,13 @@ extern "C" int cosm_server_create(const cosm_server_config *cfg, cosm_server **o
         delete s;
         return fail(COSM_ERR_CUDA, "server device setup failed");
     }
-    s->worker = std::thread(worker_main, s);
+    try {
+        s->worker = std::thread(worker_main, s);
+    } catch (const std::system_error &) {
+        cudaStreamDestroy(s->st);
+        delete s;
+        return fail(COSM_ERR_NOMEM, "the server's thread could not be created");
+    }
     *out = s;
     return COSM_OK;
 }

@@ -187,3 +187,33 @@ def test_failed_batch_run_ends_the_batch_state(cosm):
     b.get_state(1)
     b.close()
     assert report(cosm)["bad"] == 0
+
+
+def test_host_threads_that_cannot_be_created(fake_path):
+    # the calling thread does the work; in a process of its own, as an escaping
+    # exception would end it
+    code = """
+import sys; sys.path[:0] = [%r, %r]
+import test_host_runtime_cpu as T, instances
+cosm = T.load_fake(%r)
+insts = [g() for g in T.GRAPHS.values()] * 3
+lib = cosm.lib()
+lib.fake_fail_threads(1)
+b = cosm.Batch(insts)
+b.run(20, 4, 1)
+b.run(20, 4096, 1)
+try:
+    cosm.Server()
+    raise SystemExit("a server without its thread")
+except cosm.CosmError as e:
+    assert e.code == cosm.ERR_NOMEM
+lib.fake_fail_threads(0)
+srv = cosm.Server(max_active=16)
+lib.fake_fail_threads(1)
+ids = [srv.submit(inst, 20, 4, 1, 10 ** 9) for inst in insts]
+assert all(srv.wait(rid, 60)["status"] == cosm.EXHAUSTED for rid in ids)
+srv.close()
+T.sound(cosm)
+""" % (ROOT, os.path.join(ROOT, "tests"), fake_path)
+    done = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=120)
+    assert done.returncode == 0, done.stderr
