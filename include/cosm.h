@@ -345,7 +345,9 @@ typedef struct cosm_server cosm_server;
 /* memory_budget: device bytes the admitted requests may hold together (a
  * request's graph, phases of all its replicas, outputs, step table);
  * max_active: requests on the device at once; chunk_sweeps: sweeps each
- * active request advances per launch; threads: threads per CTA (0 = rule). */
+ * active request advances per launch; threads: threads per CTA (0 = rule; at
+ * least a warp, whole warps for edge lists; a lattice kept in registers has
+ * its patches' own count). */
 typedef struct cosm_server_config {
     int64_t memory_budget;
     int32_t max_active;

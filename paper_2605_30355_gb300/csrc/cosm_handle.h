@@ -192,6 +192,9 @@ int kernel_launch_queue(const LaunchCfg &cfg, const BatchArgs &b, cudaStream_t s
 int choose_layout(cosm_handle *h, int replicas, bool narrow_ties = false);
 // Half a thread count, in whole warps where the kernel needs them.
 inline int half_threads(int threads, bool warps) { return warps ? std::max(32, threads / 64 * 32) : threads / 2; }
+// A forced thread count (0: none) as the kernels take it: the readout scans the
+// bisectors with all lanes of a warp.
+inline int at_least_a_warp(int threads) { return threads > 0 ? std::max(32, threads) : threads; }
 // The device tables of the chosen layout (h->K, h->threads, h->shape).
 int ensure_tables(cosm_handle *h);
 int ensure_run_buffers(cosm_handle *h, int replicas);

@@ -965,7 +965,7 @@ int cosm::choose_layout(cosm_handle *h, int replicas, bool narrow_ties)
     for (int c = 0; c < h->C; ++c) max_ec = std::max(max_ec, h->off[c + 1] - h->off[c]);
     const int Ks_f32[3] = {1, 2, 4}, Ks_f16[3] = {2, 4, 8};
     const int *Ks = p.storage == COSM_F32 ? Ks_f32 : Ks_f16;
-    int forceK = env_int("COSM_K", 0), forceT = env_int("COSM_THREADS", 0);
+    int forceK = env_int("COSM_K", 0), forceT = at_least_a_warp(env_int("COSM_THREADS", 0));
     int bestK = 0, bestT = 0, bestOcc = 0;
     // 2D lattices keep their phases in registers where a patch shape fits
     // (forced threads and the cross-check switches take the passes on shared
@@ -1992,7 +1992,8 @@ static int batch_layout(cosm_batch *b, const int64_t *sweeps, const int32_t *rep
                                                                             std::min(fill, 8388608.0)))))
             return rc;
         if (b->threads && h->shape < 0) {
-            h->threads = b->threads;
+            h->threads = at_least_a_warp(b->threads);  // a tuning file may name any count
+            if (h->format >= 0) h->threads = (h->threads + 31) / 32 * 32;  // whole warps
             while (h->threads > 64 && kernel_occupancy(h, h->threads, h->smem, true) == 0)
                 h->threads = half_threads(h->threads, h->format >= 0);
         }

@@ -394,6 +394,7 @@ extern "C" int cosm_server_create(const cosm_server_config *cfg, cosm_server **o
     cosm_server *s = new (std::nothrow) cosm_server();
     if (!s) return fail(COSM_ERR_NOMEM, "host allocation failed");
     s->cfg = *cfg;
+    s->cfg.threads = at_least_a_warp(cfg->threads);
     s->t0 = std::chrono::steady_clock::now();
     if (cudaGetDevice(&s->device) != cudaSuccess ||
         cudaDeviceGetAttribute(&s->num_sms, cudaDevAttrMultiProcessorCount, s->device) != cudaSuccess ||

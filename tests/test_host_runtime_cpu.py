@@ -217,3 +217,35 @@ T.sound(cosm)
 """ % (ROOT, os.path.join(ROOT, "tests"), fake_path)
     done = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=120)
     assert done.returncode == 0, done.stderr
+
+
+def test_forced_thread_counts_are_at_least_a_warp(cosm, monkeypatch, tmp_path):
+    # the readout's scan of the bisectors takes all 32 lanes
+    lattice, edges = GRAPHS["lattice"](), GRAPHS["edges"]()
+    srv = cosm.Server(threads=8)
+    for kw in (dict(flags=cosm.NO_SCS), dict()):
+        for inst in (lattice, edges):
+            rid = srv.submit(inst, 20, 4, 1, 10 ** 9, **kw)
+            assert srv.wait(rid, 60)["status"] == cosm.EXHAUSTED
+            assert sound(cosm)["threads"] >= 32
+    srv.close()
+    monkeypatch.setenv("COSM_THREADS", "8")
+    for inst in (lattice, edges):
+        s = cosm.Solver.from_instance(inst)
+        s.run(20, 4, 1)
+        assert s.layout()["threads"] == 32
+        sound(cosm)
+    monkeypatch.delenv("COSM_THREADS")
+    cache = tmp_path / "tune.txt"
+    monkeypatch.setenv("COSM_TUNE_CACHE", str(cache))
+    for kw in (dict(flags=cosm.NO_SCS), dict()):
+        cache.write_text("")
+        b = cosm.Batch([lattice, edges], **kw)
+        b.tune(4)
+        key = cache.read_text().split()[0]
+        for threads in (8, 40):
+            cache.write_text("%s 0 %d\n" % (key, threads))
+            b.tune(4)
+            b.run(20, 4, 1)
+            assert sound(cosm)["threads"] >= 32 and b.info()["threads"] == threads
+        b.close()
