@@ -93,10 +93,11 @@ struct cosm_server {
     }
 };
 
-// Device bytes a request holds while admitted: edge records and weights,
-// vertex table, offsets, phases of all replicas (rounded to 16-byte tiles),
-// per-replica outputs, the step table, spins, block weight bits.
-static size_t estimate_footprint(const Request &r)
+// Device bytes a request holds while admitted, without what its layout adds:
+// edge records and weights, vertex tables, offsets, phases of all replicas
+// (rounded to 16-byte tiles), per-replica outputs, the step table, spins, block
+// weight bits.
+static size_t request_bytes(const Request &r)
 {
     const size_t esz = r.prm.storage == COSM_F32 ? 4 : 2;
     const size_t m = r.src.size();
@@ -104,6 +105,29 @@ static size_t estimate_footprint(const Request &r)
     // per replica: cut, bisector index, energy, bisector position (24 bytes)
     return 5 * m + 4 * (size_t)r.n + 4 * 65 + state + 24 * (size_t)r.R + 8 * (size_t)r.S + (size_t)r.n +
            (size_t)r.n / 2 + 4096;
+}
+
+// The most its layout adds: the last tile's empty places and the tiles' ready
+// words; a lattice's slot map; for a 2D torus of +-1 weights the patches'
+// weight words (at most 1,024 patches of three), else the record table -- rows
+// of 32 edges, a last one per colour part empty, the rows ahead, counts and
+// starts of 32 warps (cosm_edges.h).
+static size_t layout_bytes(const Request &r)
+{
+    const bool f32 = r.prm.storage == COSM_F32;
+    size_t spare = 0;
+    for (int K = 2; K <= (f32 ? 4 : 8); K *= 2)
+        spare = std::max(spare, (size_t)((K - r.R % K) % K) * (size_t)r.n * (f32 ? 4 : 2));
+    const size_t m = r.src.size(), slots = spare + 4 * (size_t)r.R + (r.dims[0] > 0 ? 2 * (size_t)r.n : 0);
+    int64_t wmax = 0;
+    for (int32_t w : r.w) wmax = std::max(wmax, std::abs((int64_t)w));
+    if (r.prm.flags & COSM_NO_SCS) return slots;
+    if (r.dims[0] > 0 && r.dims[2] == 0 && m == 2 * (size_t)r.n && wmax == 1 && r.color.empty())
+        return slots + 1024 * 3 * 4;
+    // one word per edge where the weight's sign is all there is to it; binary32
+    // may wrap every update, which takes two
+    const size_t words = wmax == 1 && r.n <= (1 << 15) && !f32 ? 1 : 2;
+    return slots + 4 * words * (m + 32 * kMaxColors + 32 * 32 * kRowsAhead) + 32 * 4 * (kMaxColors + 2);
 }
 
 static int admit(cosm_server *s, Request *r)
@@ -120,8 +144,16 @@ static int admit(cosm_server *s, Request *r)
     for (int k = 0; k < 3; ++k) d.dims[k] = r->dims[k];
     int rc = cosm_create(&d, &r->prm, &r->h);
     if (rc) return rc;
-    if ((rc = choose_layout(r->h, r->R)) || (rc = ensure_tables(r->h))) return rc;
-    r->h->replicas = r->R;
+    cosm_handle *h = r->h;
+    if ((rc = choose_layout(h, r->R))) return rc;
+    if (h->format >= 0 && s->cfg.threads) {
+        // a forced count, in the whole warps of a record table
+        h->threads = (s->cfg.threads + 31) / 32 * 32;
+        while (h->threads > 64 && kernel_occupancy(h, h->threads, h->smem, true) == 0)
+            h->threads = half_threads(h->threads, true);
+    }
+    if ((rc = ensure_tables(h))) return rc;
+    h->replicas = r->R;
     if ((rc = ensure_run_buffers(r->h, r->R))) return rc;
     if ((rc = upload_alpha(r->h, r->S, s->st))) return rc;
     r->h->stream = s->st;
@@ -182,13 +214,6 @@ static int run_chunk(cosm_server *s, const std::vector<Request *> &act)
         Request *r = act[(size_t)i];
         cosm_handle *h = r->h;
         h->seed = trial_seed(r->seed, r->trial);
-        int rc;
-        if (h->format >= 0 && s->cfg.threads) {
-            h->threads = (s->cfg.threads + 31) / 32 * 32;  // whole warps
-            while (h->threads > 64 && kernel_occupancy(h, h->threads, h->smem, true) == 0)
-                h->threads = half_threads(h->threads, true);
-        }
-        if ((rc = ensure_tables(h))) return rc;
         InstView v = inst_view(h);
         v.alpha_tab = h->d_alpha.p;
         v.alpha_base = 1;
@@ -462,8 +487,11 @@ extern "C" int cosm_server_submit(cosm_server *s, const cosm_graph_desc *g, cons
     r->seed = seed;
     r->target = target_cut;
     r->max_trials = max_trials;
-    r->footprint = estimate_footprint(*r);
-    if (r->footprint > (size_t)s->cfg.memory_budget) {
+    // a request that fits the budget but for its layout runs alone
+    r->footprint = request_bytes(*r);
+    const size_t budget = (size_t)s->cfg.memory_budget;
+    if (r->footprint <= budget) r->footprint = std::min(r->footprint + layout_bytes(*r), budget);
+    if (r->footprint > budget) {
         delete r;
         return fail(COSM_ERR_TOO_LARGE, "request footprint exceeds the server's memory budget");
     }

@@ -35,7 +35,7 @@ namespace {
 
 std::recursive_mutex mu;
 std::map<const char *, size_t> blocks;  // device allocations
-int64_t live = 0, fail_malloc = 0;
+int64_t live = 0, peak = 0, fail_malloc = 0;
 std::atomic<int> fail_threads{0};
 bool pending = false;     // a legacy-stream copy or set that nothing has waited for
 uintptr_t next_handle = 0x1000;
@@ -262,6 +262,7 @@ cudaError_t cudaMalloc(void **p, size_t bytes)
     *p = calloc(1, std::max<size_t>(bytes, 16));
     blocks[static_cast<char *>(*p)] = bytes;
     live += (int64_t)bytes;
+    peak = std::max(peak, live);
     return cudaSuccess;
 }
 cudaError_t cudaFree(void *p)
@@ -380,7 +381,12 @@ int cosm_probe_fp32(int32_t, double *, double *) { return COSM_ERR_CUDA; }
 // ---------------------------------------------------------------- the test's side
 void fake_fail_malloc(int64_t nth) { fail_malloc = nth; }  // the nth cudaMalloc from now on fails once
 void fake_fail_threads(int on) { fail_threads = on; }
-int64_t fake_live_bytes(void) { return live; }
+int64_t fake_peak_bytes(void)  // since the last call
+{
+    const int64_t p = peak;
+    peak = live;
+    return p;
+}
 const char *fake_message(void) { return why.c_str(); }
 void fake_report(int64_t out[8])
 {

@@ -40,7 +40,7 @@ def load_fake(path):
     cosm.LIB_PATH = path
     lib = cosm.lib()
     lib.fake_message.restype = C.c_char_p
-    lib.fake_live_bytes.restype = C.c_int64
+    lib.fake_peak_bytes.restype = C.c_int64
     lib.fake_fail_malloc.argtypes = [C.c_int64]
     return cosm
 
@@ -249,3 +249,48 @@ def test_forced_thread_counts_are_at_least_a_warp(cosm, monkeypatch, tmp_path):
             b.run(20, 4, 1)
             assert sound(cosm)["threads"] >= 32 and b.info()["threads"] == threads
         b.close()
+
+
+def _heavier(inst, wmax):
+    w = 1 + instances.Stream(9).below(wmax, inst.m)
+    return instances.Instance(inst.n, inst.src, inst.dst, np.asarray(w, np.int32), inst.dims)
+
+
+REQUESTS = {
+    "signs": lambda: instances.random_regular(6000, 3, 1),
+    "weights": lambda: _heavier(instances.sparse_gnm(5000, 60000, 2), 60),
+    "small": lambda: instances.sparse_gnm(60, 100, 3),
+    "torus": lambda: instances.torus2d(100, 100, 1),
+    "heavy torus": lambda: _heavier(instances.torus2d(60, 60, 1), 50),
+    "3D": lambda: instances.torus3d(12, 12, 14, 1),
+}
+
+
+@pytest.mark.parametrize("threads", [0, 96])
+@pytest.mark.parametrize("storage", [0, 1, 2])
+@pytest.mark.parametrize("graph", REQUESTS)
+def test_a_request_holds_no_more_than_its_footprint(cosm, graph, storage, threads):
+    inst = REQUESTS[graph]()
+    lib = cosm.lib()
+    for kw in (dict(), dict(alpha0_deg=100.0), dict(flags=cosm.NO_SCS)):
+        lib.fake_peak_bytes()
+        srv = cosm.Server(threads=threads)
+        before = lib.fake_peak_bytes()
+        srv.wait(srv.submit(inst, 50, 3, 1, 10 ** 9, storage=storage, **kw), 60)
+        held, fp = lib.fake_peak_bytes() - before, srv.stats()["peak_footprint"]
+        srv.close()
+        sound(cosm)
+        assert held <= fp + 1024, kw  # the server's own work lists of a few units
+        # what was accepted without counting the tables is accepted, alone
+        esz = 4 if storage == 0 else 2
+        base = 5 * inst.m + 4 * inst.n + 260 + 3 * (inst.n * esz + 64) + 72 + 400 + inst.n + inst.n // 2 + 4096
+        srv = cosm.Server(memory_budget=base, threads=threads)
+        ids = [srv.submit(inst, 50, 3, k, 10 ** 9, storage=storage, **kw) for k in range(2)]
+        assert all(srv.wait(rid, 60)["status"] == cosm.EXHAUSTED for rid in ids)
+        assert srv.stats()["max_concurrent"] == 1 and srv.stats()["peak_footprint"] <= base
+        srv.close()
+        srv = cosm.Server(memory_budget=base - 1)
+        with pytest.raises(cosm.CosmError) as err:
+            srv.submit(inst, 50, 3, 1, 10 ** 9, storage=storage, **kw)
+        assert err.value.code == cosm.ERR_TOO_LARGE
+        srv.close()
