@@ -314,14 +314,17 @@ int cosm_batch_get_state(cosm_batch *b, int32_t i, double *phases);
 /* Autotuner: times a short run (probe_sweeps sweeps per instance, the given
  * replica counts) of eight layouts and keeps the fastest for later runs:
  * the tile policies -- per instance the tile and threads that suit the
- * work of the whole batch, the narrowest tile, the single-instance rule for
- * the instance's own replica count, or the first rule with ties to the
- * narrower tile -- each with the per-instance thread rule, the first policy
+ * work of the whole batch, the narrowest tile of that kernel, the
+ * single-instance rule for the instance's own replica count, or the first rule
+ * with ties (modelled costs within 10 %) to the narrower tile -- each with the per-instance thread rule, the first policy
  * with 128, 256 or 512 threads per CTA forced, and the last with 256 (a
  * patch shape's thread count is not forced). Instances of one kernel, thread
  * count and occupancy form a class: one persistent launch.
  * With the environment variable COSM_TUNE_CACHE naming a file, a choice for
- * the same batch shape is read from it, and new choices are appended. */
+ * the same batch shape (sizes, colours, kernels, storage, largest weights,
+ * bisectors, wrap periods, replicas) is read from it, and new choices are
+ * appended; entries written before a policy changed its meaning are not
+ * taken. */
 int cosm_batch_tune(cosm_batch *b, const int32_t *replicas, int64_t probe_sweeps, void *stream);
 
 /* out[0] instances, out[1] classes, out[2] units, out[3] kernel launches

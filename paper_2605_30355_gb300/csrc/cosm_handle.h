@@ -187,9 +187,10 @@ int env_int(const char *name, int dflt);
 int kernel_occupancy(const cosm_handle *h, int threads, size_t smem, bool queue);
 int kernel_launch(const LaunchCfg &cfg, const KernelArgs &a, cudaStream_t st);
 int kernel_launch_queue(const LaunchCfg &cfg, const BatchArgs &b, cudaStream_t st);
-// narrow_ties: among tiles keeping as many replicas resident, the narrower
-// one (more CTAs per SM) instead of the wider one on a full GPU.
-int choose_layout(cosm_handle *h, int replicas, bool narrow_ties = false);
+// narrow_ties: among tiles keeping as many replicas resident, or of modelled
+// costs within 10 %, the narrower one (more CTAs per SM). only_K: tiles of that
+// width alone (0: any).
+int choose_layout(cosm_handle *h, int replicas, bool narrow_ties = false, int only_K = 0);
 // Half a thread count, in whole warps where the kernel needs them.
 inline int half_threads(int threads, bool warps) { return warps ? std::max(32, threads / 64 * 32) : threads / 2; }
 // A forced thread count (0: none) as the kernels take it: the readout scans the

@@ -620,12 +620,16 @@ static double shared_cost_16(int blocks, int replicas, int sms)
     return best;
 }
 
+// Modelled costs within 10 % count as a tie between a tile and one of twice
+// its width, which goes to the narrower one where narrow ties are asked for.
+static double tie_weight(bool narrow_ties, int K) { return narrow_ties ? 1.0 + 0.1 * __builtin_ctz((unsigned)K) : 1.0; }
+
 // Layout of a 2D lattice with its phases in registers (cosm_patch.cuh):
 // among the shapes and tile widths that fit, the one whose modelled time per
 // replica and sweep is lowest. Binary32 tiles hold two replicas, 16-bit ones
 // four or two. Returns false when no shape fits (the lattice then keeps its
 // phases in shared memory).
-static bool choose_patch(cosm_handle *h, int replicas, int forceK)
+static bool choose_patch(cosm_handle *h, int replicas, int forceK, bool narrow_ties)
 {
     const cosm_params &p = h->prm;
     const int BR = h->Q / h->Wd, BC = h->Wd, only = env_int("COSM_PATCH", -2);
@@ -650,7 +654,8 @@ static bool choose_patch(cosm_handle *h, int replicas, int forceK)
             const int T = (gr * gc + 31) / 32 * 32;
             const int occ = patch_occupancy(p.storage, K, s, ragged, T, smem);
             if (occ < 1) continue;
-            const double cost = patch_cost(p.storage, K, R, C, ragged, T / 32, occ, replicas, h->num_sms);
+            const double cost = patch_cost(p.storage, K, R, C, ragged, T / 32, occ, replicas, h->num_sms) *
+                                tie_weight(narrow_ties, K);
             if (cost < best) {
                 best = cost;
                 h->shape = s;
@@ -767,7 +772,7 @@ static double edges_cost(const cosm_handle *h, int K, int format, int T, int occ
 
 // Tile width and threads of an edge-list instance on record tables. False
 // when no width and thread count take them.
-static bool choose_edges(cosm_handle *h, int replicas, int forceK, int forceT)
+static bool choose_edges(cosm_handle *h, int replicas, int forceK, int forceT, bool narrow_ties)
 {
     const cosm_params &p = h->prm;
     const int Ts[8] = {64, 128, 192, 256, 384, 512, 768, 1024};
@@ -781,7 +786,7 @@ static bool choose_edges(cosm_handle *h, int replicas, int forceK, int forceT)
             const int T = forceT ? forceT : Ts[k];
             const int occ = edges_occupancy(p.storage, K, format, T, smem);
             if (occ < 1) continue;
-            const double cost = edges_cost(h, K, format, T, occ, replicas);
+            const double cost = edges_cost(h, K, format, T, occ, replicas) * tie_weight(narrow_ties, K);
             if (cost < best) {
                 best = cost;
                 h->K = K;
@@ -956,7 +961,7 @@ int cosm::ensure_tables(cosm_handle *h)
 
 // Replicas per CTA (K) and threads per CTA: maximise resident replicas per
 // SM (COSM_K / COSM_THREADS override for experiments).
-int cosm::choose_layout(cosm_handle *h, int replicas, bool narrow_ties)
+int cosm::choose_layout(cosm_handle *h, int replicas, bool narrow_ties, int only_K)
 {
     const cosm_params &p = h->prm;
     const int mode = h->mode;
@@ -965,7 +970,7 @@ int cosm::choose_layout(cosm_handle *h, int replicas, bool narrow_ties)
     for (int c = 0; c < h->C; ++c) max_ec = std::max(max_ec, h->off[c + 1] - h->off[c]);
     const int Ks_f32[3] = {1, 2, 4}, Ks_f16[3] = {2, 4, 8};
     const int *Ks = p.storage == COSM_F32 ? Ks_f32 : Ks_f16;
-    int forceK = env_int("COSM_K", 0), forceT = at_least_a_warp(env_int("COSM_THREADS", 0));
+    int forceK = env_int("COSM_K", only_K), forceT = at_least_a_warp(env_int("COSM_THREADS", 0));
     int bestK = 0, bestT = 0, bestOcc = 0;
     // 2D lattices keep their phases in registers where a patch shape fits
     // (forced threads and the cross-check switches take the passes on shared
@@ -976,7 +981,7 @@ int cosm::choose_layout(cosm_handle *h, int replicas, bool narrow_ties)
     // available as cross-checks)
     h->shape = -1;
     if (mode == MODE_LATTICE2D_ && !forceT && !std::getenv("COSM_SCALAR_F32") && !std::getenv("COSM_SINGLE_BLOCKS") &&
-        choose_patch(h, replicas, forceK)) {
+        choose_patch(h, replicas, forceK, narrow_ties)) {
         h->block_pairs = false;
         h->staged = false;
         const size_t esz = p.storage == COSM_F32 ? 4 : 2;
@@ -984,7 +989,7 @@ int cosm::choose_layout(cosm_handle *h, int replicas, bool narrow_ties)
         h->format = -1;
         return COSM_OK;
     }
-    if (mode == MODE_GENERAL_ && choose_edges(h, replicas, forceK, forceT)) {
+    if (mode == MODE_GENERAL_ && choose_edges(h, replicas, forceK, forceT, narrow_ties)) {
         h->block_pairs = false;
         h->staged = false;
         const size_t esz = p.storage == COSM_F32 ? 4 : 2;
@@ -1919,7 +1924,8 @@ extern "C" int cosm_batch_create(int32_t count, const cosm_graph_desc *graphs, c
 // up to 20,000: 9.0 / 8.7 / 9.1). Policy 1: the narrowest tile of the storage
 // type. Policy 2: the single-instance rule with the instance's own replica
 // count. Policy 3: as policy 0 with ties to the narrower tile (more CTAs per
-// SM, whose barriers and record loads overlap). Kernels without a fitted cost
+// SM, whose barriers and record loads overlap; modelled costs within 10 % are
+// a tie). Kernels without a fitted cost
 // (plain records, lattices on shared memory) score policies 0, 1 and 3 as if
 // the run filled every CTA slot.
 static int batch_instance_layout(cosm_batch *b, cosm_handle *h, int32_t replicas, int32_t fill)
@@ -1928,20 +1934,9 @@ static int batch_instance_layout(cosm_batch *b, cosm_handle *h, int32_t replicas
     if (b->policy == 2) return choose_layout(h, replicas);
     if ((rc = choose_layout(h, fill, b->policy == 3))) return rc;
     if (h->shape < 0 && h->format < 0 && (rc = choose_layout(h, 1 << 23, b->policy == 3))) return rc;
-    if (b->policy == 1 && h->shape < 0 && h->K != (h->prm.storage == COSM_F32 ? 1 : 2)) {
-        const int Kmin = h->prm.storage == COSM_F32 ? 1 : 2;
-        const size_t esz = h->prm.storage == COSM_F32 ? 4 : 2;
-        h->K = Kmin;
-        h->format = record_format(h, Kmin);
-        h->block_pairs = false;
-        h->staged = false;
-        h->smem = sweep_smem_bytes(h->prm.storage, Kmin, h->g.n, h->prm.n_bisectors, h->mode);
-        h->tile_stride = (int64_t)(((size_t)h->g.n * Kmin * esz + 15) / 16 * 16 / esz);
-        // the narrow tile's kernel may allow fewer threads per CTA
-        while (h->threads > 64 && kernel_occupancy(h, h->threads, h->smem, true) == 0)
-            h->threads = half_threads(h->threads, h->format >= 0);
-        h->occupancy = kernel_occupancy(h, h->threads, h->smem, true);
-    }
+    // two replicas are the least a lattice in registers has
+    const int narrowest = h->prm.storage == COSM_F32 && h->shape < 0 ? 1 : 2;
+    if (b->policy == 1 && h->K != narrowest) return choose_layout(h, fill, false, narrowest);
     return COSM_OK;
 }
 
@@ -2229,7 +2224,12 @@ extern "C" int cosm_batch_tune(cosm_batch *b, const int32_t *replicas, int64_t p
         const cosm_handle *h = b->hs[i];
         mix((uint64_t)h->g.n); mix((uint64_t)h->g.m); mix((uint64_t)h->C); mix((uint64_t)h->mode);
         mix((uint64_t)h->prm.storage); mix((uint64_t)replicas[i]);
+        // what decides an instance's kernel and record format besides
+        mix((uint64_t)h->wmax); mix((uint64_t)h->prm.n_bisectors);
+        mix((uint64_t)wrap_period(h->prm.alpha0_deg, h->prm.dwt_ratio, h->prm.dwt_period, h->prm.flags, h->mode,
+                                  h->prm.storage, h->wbound));
     }
+    mix(2);  // the policies' meaning: an entry chosen under another one is not taken
     const char *cache = std::getenv("COSM_TUNE_CACHE");
     if (cache) {
         FILE *f = std::fopen(cache, "r");

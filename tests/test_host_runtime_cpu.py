@@ -294,3 +294,35 @@ def test_a_request_holds_no_more_than_its_footprint(cosm, graph, storage, thread
             srv.submit(inst, 50, 3, 1, 10 ** 9, storage=storage, **kw)
         assert err.value.code == cosm.ERR_TOO_LARGE
         srv.close()
+
+
+def test_tile_policies_differ_and_tuning_keys_name_what_decides_them(cosm, monkeypatch, tmp_path):
+    cache = tmp_path / "tune.txt"
+    monkeypatch.setenv("COSM_TUNE_CACHE", str(cache))
+
+    def key(insts, **kw):
+        cache.write_text("")
+        b = cosm.Batch(insts, **kw)
+        b.tune(64)
+        return cache.read_text().split()[0], b
+
+    edges = [instances.sparse_gnm(n, 5 * n // 2, n) for n in (300, 1000, 2500, 5000, 9000)]
+    for insts, kw, least in ((edges, dict(), 1), (edges, dict(storage=1), 2), (edges, dict(storage=2), 2),
+                             ([instances.torus2d(40, 40, 1)], dict(), 2),
+                             ([instances.torus2d(40, 40, 1)], dict(storage=2), 2)):
+        k, b = key(insts, **kw)
+        widths = {}
+        for policy in range(4):
+            cache.write_text("%s %d 0\n" % (k, policy))
+            b.tune(64)
+            b.run(50, 64, 1)
+            sound(cosm)
+            widths[policy] = [b.layout(i)["K"] for i in range(len(insts))]
+        b.close()
+        assert widths[1] == [least] * len(insts)
+        assert all(x <= y for x, y in zip(widths[3], widths[0]))
+        assert insts is not edges or widths[3] != widths[0], widths
+    base, _ = key(edges)
+    heavier, _ = key(edges[:-1] + [_heavier(edges[-1], 40)])
+    others = [key(edges, **kw)[0] for kw in (dict(n_bisectors=7), dict(alpha0_deg=120.0))]
+    assert len({base, heavier, *others}) == 4
