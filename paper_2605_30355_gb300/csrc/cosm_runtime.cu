@@ -1824,8 +1824,16 @@ struct BatchClass {
     int32_t unit0, units;
 };
 
+// What an instance's layout in a batch was chosen for, and its CTAs per SM: a
+// run with the same ones keeps the layout (choosing it asks the driver for the
+// occupancy of up to 24 kernel configurations).
+struct BatchChoice {
+    int32_t replicas = 0, fill = 0, policy = -1, threads = -1, occupancy = 0;
+};
+
 struct cosm_batch {
     std::vector<cosm_handle *> hs;
+    std::vector<BatchChoice> chosen;  // per instance; empty after a run that failed
     std::vector<BatchClass> classes;
     std::vector<BatchUnit> h_units;
     DevBuf<BatchUnit> d_units;
@@ -1977,20 +1985,25 @@ static int batch_layout(cosm_batch *b, const int64_t *sweeps, const int32_t *rep
     const int n = (int)b->hs.size();
     std::vector<InstView> views((size_t)n);
     std::vector<BatchFinal> fins((size_t)n);
+    b->chosen.resize((size_t)n);
     double total = 0.0;  // edge updates of the run
     for (int i = 0; i < n; ++i) total += (double)b->hs[(size_t)i]->g.m * (double)replicas[i] * (double)sweeps[i];
     for (int i = 0; i < n; ++i) {
         cosm_handle *h = b->hs[(size_t)i];
         int rc;
-        const double fill = 0.6 * total / ((double)h->g.m * (double)sweeps[i]);
-        if ((rc = batch_instance_layout(b, h, replicas[i], (int32_t)std::max((double)replicas[i],
-                                                                            std::min(fill, 8388608.0)))))
-            return rc;
-        if (b->threads && h->shape < 0) {
-            h->threads = at_least_a_warp(b->threads);  // a tuning file may name any count
-            if (h->format >= 0) h->threads = (h->threads + 31) / 32 * 32;  // whole warps
-            while (h->threads > 64 && kernel_occupancy(h, h->threads, h->smem, true) == 0)
-                h->threads = half_threads(h->threads, h->format >= 0);
+        const double share = 0.6 * total / ((double)h->g.m * (double)sweeps[i]);
+        const int32_t fill = (int32_t)std::max((double)replicas[i], std::min(share, 8388608.0));
+        BatchChoice &was = b->chosen[(size_t)i];
+        if (was.replicas != replicas[i] || was.fill != fill || was.policy != b->policy || was.threads != b->threads) {
+            was = BatchChoice();
+            if ((rc = batch_instance_layout(b, h, replicas[i], fill))) return rc;
+            if (b->threads && h->shape < 0) {
+                h->threads = at_least_a_warp(b->threads);  // a tuning file may name any count
+                if (h->format >= 0) h->threads = (h->threads + 31) / 32 * 32;  // whole warps
+                while (h->threads > 64 && kernel_occupancy(h, h->threads, h->smem, true) == 0)
+                    h->threads = half_threads(h->threads, h->format >= 0);
+            }
+            was = BatchChoice{replicas[i], fill, b->policy, b->threads, kernel_occupancy(h, h->threads, h->smem, true)};
         }
         h->replicas = replicas[i];
         h->seed = seeds[i];
@@ -2019,7 +2032,7 @@ static int batch_layout(cosm_batch *b, const int64_t *sweeps, const int32_t *rep
     for (int i = 0; i < n; ++i) {
         const cosm_handle *h = b->hs[(size_t)i];
         const Key k{h->prm.storage, h->K, h->mode, h->shape, h->shape >= 0 && h->ragged, h->format, h->threads,
-                    kernel_occupancy(h, h->threads, h->smem, true)};
+                    b->chosen[(size_t)i].occupancy};
         int c = -1;
         for (size_t q = 0; q < keys.size() && c < 0; ++q) {
             const Key &o = keys[q];
@@ -2131,6 +2144,7 @@ extern "C" int cosm_batch_run(cosm_batch *b, const int64_t *sweeps, const int32_
         // some instances have a new layout: the last run's states and results end here
         for (cosm_handle *h : b->hs) h->have_state = h->have_result = false;
         b->have_result = false;
+        b->chosen.clear();
         return rc;
     }
     std::vector<int64_t> sig;

@@ -37,6 +37,7 @@ std::recursive_mutex mu;
 std::map<const char *, size_t> blocks;  // device allocations
 int64_t live = 0, peak = 0, fail_malloc = 0;
 std::atomic<int> fail_threads{0};
+std::atomic<int64_t> queries{0};  // of occupancies, since the last report
 bool pending = false;     // a legacy-stream copy or set that nothing has waited for
 uintptr_t next_handle = 0x1000;
 struct Report {
@@ -63,6 +64,7 @@ void launched(void *stream)
 }
 int model_occupancy(int threads, size_t smem)
 {
+    ++queries;
     if (threads < 1 || threads > 1024 || smem > 227 * 1024) return 0;
     return (int)std::min<size_t>(1024 / (size_t)((threads + 31) / 32 * 32), 228 * 1024 / (smem + 1024));
 }
@@ -388,6 +390,7 @@ int64_t fake_peak_bytes(void)  // since the last call
     return p;
 }
 const char *fake_message(void) { return why.c_str(); }
+int64_t fake_queries(void) { return queries.exchange(0); }
 void fake_report(int64_t out[8])
 {
     memcpy(out, &rep, sizeof(rep));

@@ -326,3 +326,30 @@ def test_tile_policies_differ_and_tuning_keys_name_what_decides_them(cosm, monke
     heavier, _ = key(edges[:-1] + [_heavier(edges[-1], 40)])
     others = [key(edges, **kw)[0] for kw in (dict(n_bisectors=7), dict(alpha0_deg=120.0))]
     assert len({base, heavier, *others}) == 4
+
+
+def test_a_repeated_batch_run_keeps_its_layouts(cosm):
+    lib = cosm.lib()
+    lib.fake_queries.restype = C.c_int64
+    insts = [g() for g in GRAPHS.values()] * 4
+    b = cosm.Batch(insts)
+    b.run(20, 4, 1)
+    first, info = lib.fake_queries(), b.info()
+    b.run(20, 4, 2)
+    assert lib.fake_queries() == info["classes"] < first and b.info()["graphs_built"] == 1
+    sound(cosm)
+    b.run(20, 700, 2)  # other replicas: chosen again
+    assert lib.fake_queries() > info["classes"]
+    other = [b.layout(i) for i in range(8)]
+    c = cosm.Batch(insts)
+    c.run(20, 700, 2)
+    assert other == [c.layout(i) for i in range(8)]
+    sound(cosm)
+    lib.fake_fail_malloc(1)
+    with pytest.raises(cosm.CosmError):
+        b.run(20, 40000, 2)
+    b.run(20, 700, 2)
+    assert other == [b.layout(i) for i in range(8)]
+    b.close()
+    c.close()
+    sound(cosm)
