@@ -605,9 +605,11 @@ int patch_call(const PatchCall &c)
 template <typename Store, int K>
 int patch_dispatch(const PatchCall &c)
 {
-#define PATCH_CASE(I, R, C)                                                              \
-    if (c.shape == (I))                                                                  \
-        return c.ragged ? patch_call<Store, K, R, C, (R) * (C) != 1>(c) : patch_call<Store, K, R, C, false>(c);
+    constexpr bool float16 = sizeof(Store) == 2 && !std::is_same<Store, uint16_t>::value;
+#define PATCH_CASE(I, R, C)                                                                  \
+    if constexpr (patch_built(float16, K, R, C))                                             \
+        if (c.shape == (I))                                                                  \
+            return c.ragged ? patch_call<Store, K, R, C, (R) * (C) != 1>(c) : patch_call<Store, K, R, C, false>(c);
     COSM_PATCH_SHAPES(PATCH_CASE)
 #undef PATCH_CASE
     return c.what == PatchCall::OCCUPANCY ? 0 : -1;

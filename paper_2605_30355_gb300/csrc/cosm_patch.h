@@ -24,6 +24,9 @@ constexpr int patch_max_threads(int R, int C, int site_bytes)
     return regs > 96 ? 512 : regs > 80 ? 640 : regs > 64 ? 768 : 1024;
 }
 
+// Four 16-bit floats per site spill above 2 x 2 blocks: no such kernel.
+constexpr bool patch_built(bool float16, int K, int R, int C) { return !(float16 && K == 4 && R * C > 4); }
+
 struct PatchCall {
     enum What { OCCUPANCY, LAUNCH } what;
     int shape;

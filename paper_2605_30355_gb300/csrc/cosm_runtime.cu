@@ -643,8 +643,7 @@ static bool choose_patch(cosm_handle *h, int replicas, int forceK, bool narrow_t
         const size_t smem = sweep_smem_bytes(p.storage, K, h->g.n, p.n_bisectors, MODE_LATTICE2D_);
         for (int s = 0; s < kPatchShapes; ++s) {
             if (only >= 0 && s != only) continue;
-            // four 16-bit floats per site: patches above 2x2 blocks spill
-            if (only < 0 && f16 && K == 4 && kPatchR[s] * kPatchC[s] > 4) continue;
+            if (!patch_built(f16, K, kPatchR[s], kPatchC[s])) continue;
             const int R = kPatchR[s], C = kPatchC[s], NE = 2 * R + 2 * C - 1;
             int gr, gc, fr, fc;
             if (!split_side(BR, R, &gr, &fr) || !split_side(BC, C, &gc, &fc)) continue;
