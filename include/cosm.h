@@ -428,6 +428,15 @@ void cosm_server_destroy(cosm_server *s);
  * out[5] CTAs in the last launch, out[6] kernel launches in the last run. */
 int cosm_layout(cosm_handle *h, int32_t out[8]);
 
+/* The sweep kernel of the handle's layout: out[0] the patch shape of a 2D
+ * lattice kept in registers (0 .. 5: 2 x 5, 2 x 4, 2 x 3, 2 x 2, 1 x 2, 1 x 1
+ * blocks per thread), -1 where phases stay in shared memory; out[1] 1 where
+ * the shape does not divide the lattice; out[2] the record format of an edge
+ * list (0 sign and slots in a word, 1 weight and slots in a word, 2 two words;
+ * plus 4 where every update is wrapped), -1 without a record table; out[3]
+ * reserved (0). */
+int cosm_layout_form(cosm_handle *h, int32_t out[4]);
+
 /* ---- edge colourings (host only; Alg. 1 line 1) ------------------------ */
 
 /* Greedy colouring of Section II-B: edges in the given order each take the

@@ -58,7 +58,7 @@ EXPORTS = (
     "cosm_server_stats", "cosm_server_destroy", "cosm_last_error", "cosm_get_replica_energies",
     "cosm_get_replica_bisectors", "cosm_get_trace", "cosm_qubo_to_ising", "cosm_probe_fp32",
     "cosm_run_range", "cosm_get_success", "cosm_export_state", "cosm_import_state",
-    "cosm_set_wait_limit", "cosm_inject_fault", "cosm_batch_layout",
+    "cosm_set_wait_limit", "cosm_inject_fault", "cosm_batch_layout", "cosm_layout_form",
 )
 
 
@@ -122,6 +122,7 @@ def _load():
         "cosm_readout": (C.c_int, [P, P]),
         "cosm_solve": (C.c_int, [P, P, i64, i32, u64, P, P, P, P]),
         "cosm_layout": (C.c_int, [P, P]),
+        "cosm_layout_form": (C.c_int, [P, P]),
         "cosm_color_greedy": (C.c_int, [i32, i64, P, P, P, P]),
         "cosm_color_misra_gries": (C.c_int, [i32, i64, P, P, P, P]),
         "cosm_color_torus2d": (C.c_int, [i32, i32, i64, P, P, P]),
@@ -361,6 +362,14 @@ class Solver:
         _check(_lib.cosm_layout(self._h, out))
         keys = ("K", "threads", "smem", "occupancy", "lattice", "grid", "launches", "colors")
         return dict(zip(keys, list(out)))
+
+
+    def layout_form(self):
+        """The sweep kernel of the layout (cosm_layout_form): patch shape or
+        record format, -1 where there is none."""
+        out = (C.c_int32 * 4)()
+        _check(_lib.cosm_layout_form(self._h, out))
+        return dict(zip(("shape", "ragged", "format"), list(out)))
 
 
 class Batch:

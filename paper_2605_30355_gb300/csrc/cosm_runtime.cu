@@ -1788,6 +1788,16 @@ extern "C" int cosm_layout(cosm_handle *h, int32_t out[8])
     return COSM_OK;
 }
 
+extern "C" int cosm_layout_form(cosm_handle *h, int32_t out[4])
+{
+    if (!h || !out) return fail(COSM_ERR_INVALID_ARG, "NULL argument");
+    out[0] = h->shape;
+    out[1] = h->shape >= 0 && h->ragged;
+    out[2] = h->format;
+    out[3] = 0;
+    return COSM_OK;
+}
+
 extern "C" int cosm_solve(const cosm_graph_desc *g, const cosm_params *p, int64_t sweeps, int32_t replicas,
                           uint64_t seed, int64_t *best_cut, int64_t *energy, int8_t *spins,
                           int64_t *replica_cuts)

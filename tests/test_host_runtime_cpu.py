@@ -328,6 +328,49 @@ def test_tile_policies_differ_and_tuning_keys_name_what_decides_them(cosm, monke
     assert len({base, heavier, *others}) == 4
 
 
+def _weighted(n, m, wmax, seed):
+    inst = instances.sparse_gnm(n, m, seed, wmax=wmax)
+    w = np.array(inst.w, np.int32)
+    w[:2] = wmax, -wmax  # the extremes are there
+    return instances.Instance(inst.n, inst.src, inst.dst, w)
+
+
+# (vertices, largest weight, storage, tile width) -> format: both sides of every
+# limit (2^14 and 2^15 slots, the weights a code or two words hold, every
+# update wrapped)
+FORMATS = [
+    ((5, 1, 0, 1), 0), ((700, 1, 0, 4), 0), ((700, 1, 1, 8), 0), ((700, 1, 2, 8), 0),
+    ((1 << 15, 1, 0, 1), 0), ((1 << 15, 1, 1, 2), 0), ((1 << 15, 1, 2, 2), 0),
+    (((1 << 15) + 1, 1, 0, 1), 2), (((1 << 15) + 1, 1, 1, 2), 2), (((1 << 15) + 1, 1, 2, 2), 2),
+    ((700, 2, 0, 1), 2), ((700, 2, 1, 2), 2), ((700, 3, 0, 2), 1), ((700, 3, 1, 4), 1), ((700, 3, 2, 4), 1),
+    ((700, 4, 0, 2), 2), ((700, 4, 1, 4), 2), ((700, 4, 2, 4), 2),
+    ((700, 7, 0, 4), 1), ((700, 7, 1, 8), 1), ((700, 7, 2, 8), 1), ((700, 8, 0, 4), 2), ((700, 8, 2, 8), 2),
+    ((1 << 14, 3, 0, 2), 1), ((1 << 14, 3, 1, 4), 1), (((1 << 14) + 1, 3, 0, 2), 2), (((1 << 14) + 1, 3, 2, 4), 2),
+    ((14000, 7, 0, 4), 1), ((14000, 7, 1, 8), 1),  # byte offsets close to 2^18
+    ((56000, 63, 0, 1), 2), ((56000, 63, 1, 2), 2), ((56000, 127, 2, 2), 2),
+    ((700, 63, 0, 2), 2), ((700, 64, 0, 2), -1), ((700, 64, 3, 2), -1), ((700, 127, 2, 4), 2),
+]
+
+
+@pytest.mark.parametrize("case,fmt", FORMATS)
+def test_record_tables_hold_every_edge(cosm, monkeypatch, case, fmt):
+    n, wmax, storage, K = case
+    inst = _weighted(n, min(n + n // 4, n * (n - 1) // 2), wmax, n)
+    monkeypatch.setenv("COSM_K", str(K))
+    for kw, each in ((dict(alpha0_deg=0.1), 0), (dict(alpha0_deg=170.0, dwt_period=1), 4 if storage == 0 else 0)):
+        want = fmt + each if fmt >= 0 else -1
+        if fmt == 0 and each:
+            want = 4 + (1 if K > 1 and n <= 1 << 14 else 2)
+        for threads in ("32", "96", "1024"):
+            monkeypatch.setenv("COSM_THREADS", threads)
+            s = cosm.Solver(inst.n, inst.src, inst.dst, inst.w, storage=storage, **kw)
+            s.run(3, 2 * K + 1, 1)
+            r = sound(cosm)
+            assert r["format"] == want and r["K"] == K and r["threads"] == int(threads)
+            assert s.layout_form()["format"] == want
+            s.close()
+
+
 def test_a_repeated_batch_run_keeps_its_layouts(cosm):
     lib = cosm.lib()
     lib.fake_queries.restype = C.c_int64
