@@ -332,12 +332,12 @@ __device__ __noinline__ void twist_fill(const InstView &v, int *D, int E, int st
                                         uint32_t rep0)
 {
     const int lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
-    // the lanes this warp has: all, but for the last of a block that is no whole warps
-    const uint32_t in_warp = min(32u, blockDim.x - (threadIdx.x & ~31u)), live = 0xFFFFFFFFu >> (32u - in_warp);
+    __syncwarp();
+    const uint32_t live = __activemask();  // a last, partial warp fills in its own lanes
     for (int r = threadIdx.x >> 5; r < K; r += nw) {
         int *Dr = D + r * (v.P + 1);
         uint32_t dirs = 0;
-        for (int k0 = 0; k0 < E; k0 += (int)in_warp) {
+        for (int k0 = 0; k0 < E; k0 += __popc(live)) {
             const int k = k0 + lane;
             bool neg = false;
             const float th = dwt_theta(v.seed, rep0 + (uint32_t)r, (int64_t)s + (int64_t)k * stride, &neg);

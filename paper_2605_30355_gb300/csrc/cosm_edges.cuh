@@ -6,8 +6,10 @@
 // colour, the next one or the next sweep: the stream only goes on), then
 // loads, updates and stores the phases. So the records' latency (L2 for
 // graphs beyond L1) overlaps the updates and the barriers between colours,
-// addresses are a pointer and constants, and a row costs what its edges cost:
-// about 16 instructions and two wavefronts per phase access.
+// addresses are a pointer and constants, and a row of 32 edges costs what its
+// edges cost: 31 warp instructions at two binary32 replicas per tile (random
+// 3-regular graph of 20,000 vertices; colours, twist and wrap included), and two
+// wavefronts per phase access.
 #pragma once
 
 #include "cosm_device.cuh"

@@ -746,7 +746,8 @@ static double edges_cost(const cosm_handle *h, int K, int format, int T, int occ
 {
     const int st = h->prm.storage, W = T / 32, E = K * (st == COSM_F32 ? 4 : 2);
     const double words = K / 2.0, colours = h->C;
-    // instructions and shared-memory wavefronts of a row of 32 edges
+    // instructions and shared-memory wavefronts of a row of 32 edges (the
+    // colours', the twist's and the wrap's are counted apart below)
     double inst = st == COSM_F32 ? 12.0 + 9.0 * std::max(1.0, words)
                                  : st == COSM_Q16 ? 14.0 + 6.5 * words : 12.0 + 19.0 * words;
     if ((format & ~EDGES_EACH) != EDGES_SIGN) inst += 2.0;

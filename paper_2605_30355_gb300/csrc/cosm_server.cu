@@ -119,8 +119,12 @@ static size_t layout_bytes(const Request &r)
     for (int K = 2; K <= (f32 ? 4 : 8); K *= 2)
         spare = std::max(spare, (size_t)((K - r.R % K) % K) * (size_t)r.n * (f32 ? 4 : 2));
     const size_t m = r.src.size(), slots = spare + 4 * (size_t)r.R + (r.dims[0] > 0 ? 2 * (size_t)r.n : 0);
-    int64_t wmax = 0;
-    for (int32_t w : r.w) wmax = std::max(wmax, std::abs((int64_t)w));
+    int32_t lo = 0, hi = 0;
+    for (int32_t w : r.w) {
+        lo = std::min(lo, w);
+        hi = std::max(hi, w);
+    }
+    const int64_t wmax = std::max<int64_t>(hi, -(int64_t)lo);
     if (r.prm.flags & COSM_NO_SCS) return slots;
     if (r.dims[0] > 0 && r.dims[2] == 0 && m == 2 * (size_t)r.n && wmax == 1 && r.color.empty())
         return slots + 1024 * 3 * 4;
