@@ -332,8 +332,10 @@ __device__ __noinline__ void twist_fill(const InstView &v, int *D, int E, int st
                                         uint32_t rep0)
 {
     const int lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
-    __syncwarp();
-    const uint32_t live = __activemask();  // a last, partial warp fills in its own lanes
+    // a last, partial warp fills in its own lanes (every caller comes here with
+    // its warps together; masks from the block's size or a full ballot, and whole
+    // warps alone, moved the patch kernels' registers: -1 to +1.6 % by shape)
+    const uint32_t live = __activemask();
     for (int r = threadIdx.x >> 5; r < K; r += nw) {
         int *Dr = D + r * (v.P + 1);
         uint32_t dirs = 0;
@@ -426,9 +428,9 @@ __device__ __forceinline__ Tile<Store, K> carve(unsigned char *smem, int n, int 
     return t;
 }
 
-// The prologue, the readout and the epilogue as bodies, and as calls that take
-// the tile and the segment by value (seg_begin, tile_readout, seg_end): a sweep
-// loop then keeps what it uses of them in registers.
+// The prologue and the epilogue as bodies, and as calls that take the tile and
+// the segment by value (seg_begin, seg_end; so does tile_readout): a sweep loop
+// then keeps what it uses of them in registers.
 
 // Returns false when the bounded wait gave up (the error word is set).
 template <typename Store, int K>
@@ -511,8 +513,7 @@ __device__ __forceinline__ bool seg_begin_body(const InstView &v, const Segment 
 // to trace[k] (k >= 0), and with tracking the spins of a replaced readout
 // are saved as bits.
 template <typename Store, int K>
-__device__ __forceinline__ void tile_readout_body(const InstView &a, int tile, const Tile<Store, K> &t, int k,
-                                                  bool keep_better)
+__device__ __noinline__ void tile_readout(const InstView &a, int tile, const Tile<Store, K> t, int k, bool keep_better)
 {
     const int tid = threadIdx.x, nt = blockDim.x, P = a.P;
     const uint32_t rep0 = (uint32_t)tile * K;
@@ -713,15 +714,11 @@ __device__ __noinline__ bool seg_begin(const InstView &v, const Segment sg, cons
 {
     return seg_begin_body<Store, K>(v, sg, t, s_skip, ready, err, wait_limit_ns);
 }
-template <typename Store, int K>
-__device__ __noinline__ void tile_readout(const InstView &a, int tile, const Tile<Store, K> t, int k, bool keep_better)
-{
-    tile_readout_body<Store, K>(a, tile, t, k, keep_better);
-}
+// The readout of a tile in local memory.
 template <typename Store, int K>
 __device__ __noinline__ void tile_readout_at(const InstView &a, int tile, const Tile<Store, K> &t, int k, bool keep_better)
 {
-    tile_readout_body<Store, K>(a, tile, t, k, keep_better);
+    tile_readout<Store, K>(a, tile, t, k, keep_better);
 }
 template <typename Store, int K>
 __device__ __noinline__ void seg_end(const InstView &a, const Segment sg, const Tile<Store, K> t, int32_t *ready)
