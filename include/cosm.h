@@ -347,8 +347,9 @@ typedef struct cosm_server cosm_server;
 
 /* memory_budget: device bytes the admitted requests may hold together (a
  * request's graph, phases of all its replicas, outputs, step table and the
- * most that its kernel's tables and a part-filled tile can add; a request that
- * exceeds the budget only by the latter is admitted alone);
+ * most that its kernel's tables and a part-filled tile can add, until it is
+ * admitted and what it holds is known; a request that exceeds the budget only by
+ * the latter is admitted alone);
  * max_active: requests on the device at once; chunk_sweeps: sweeps each
  * active request advances per launch; threads: threads per CTA (0 = rule; at
  * least a warp, whole warps for edge lists; a lattice kept in registers has

@@ -199,6 +199,8 @@ inline int at_least_a_warp(int threads) { return threads > 0 ? std::max(32, thre
 // The device tables of the chosen layout (h->K, h->threads, h->shape).
 int ensure_tables(cosm_handle *h);
 int ensure_run_buffers(cosm_handle *h, int replicas);
+// Device bytes of a handle's graph, tables and run buffers.
+size_t device_bytes(const cosm_handle *h);
 InstView inst_view(cosm_handle *h);
 int upload_alpha(cosm_handle *h, int64_t S, cudaStream_t st);
 int launch_finalize(cosm_handle *h, cudaStream_t st);

@@ -1093,6 +1093,17 @@ int cosm::ensure_run_buffers(cosm_handle *h, int replicas)
     return COSM_OK;
 }
 
+size_t cosm::device_bytes(const cosm_handle *h)
+{
+    const auto sum = [](const auto &...b) { return (size_t(0) + ... + (b.cap * sizeof(*b.p))); };
+    size_t bytes = sum(h->d_ij, h->d_w, h->d_orig, h->d_slot, h->d_off, h->d_wnib, h->d_h, h->d_hlist, h->d_state, h->d_cut,
+                       h->d_bestp, h->d_alpha, h->d_segs, h->d_segoff, h->d_ready, h->d_err, h->d_best, h->d_spins,
+                       h->d_energy, h->d_bisB, h->d_trace, h->d_bits, h->d_qbuf, h->d_delta, h->d_items, h->d_stage);
+    for (const auto &b : h->d_pwt) bytes += sum(b);
+    for (const auto &t : h->tables) bytes += sum(t->rec, t->counts, t->starts);
+    return bytes;
+}
+
 int32_t cosm::wrap_period(double alpha0_deg, double dwt_ratio, int dwt_period, int flags, int mode, int storage,
                           int64_t wbound)
 {

@@ -7,6 +7,7 @@ import importlib.util
 import os
 import subprocess
 import sys
+import time
 
 import numpy as np
 import pytest
@@ -326,6 +327,33 @@ def test_tile_policies_differ_and_tuning_keys_name_what_decides_them(cosm, monke
     heavier, _ = key(edges[:-1] + [_heavier(edges[-1], 40)])
     others = [key(edges, **kw)[0] for kw in (dict(n_bisectors=7), dict(alpha0_deg=120.0))]
     assert len({base, heavier, *others}) == 4
+
+
+def test_an_admitted_request_counts_what_it_holds(cosm):
+    # two requests whose bounds exceed the budget, not what they hold: the
+    # second joins the first once that is admitted
+    inst, sweeps = REQUESTS["torus"](), 30000
+    lib = cosm.lib()
+
+    def running(srv, count):
+        end = time.monotonic() + 30
+        while srv.stats()["active"] < count:
+            assert time.monotonic() < end
+
+    srv = cosm.Server(chunk_sweeps=1)
+    rid = srv.submit(inst, sweeps, 4, 1, 10 ** 9, storage=1)
+    running(srv, 1)
+    st = srv.stats()
+    held, bound = st["footprint"], st["peak_footprint"]
+    assert 0 < held < bound
+    srv.close()
+    srv = cosm.Server(chunk_sweeps=1, memory_budget=held + bound)
+    for k in range(2):
+        srv.submit(inst, sweeps, 4, k, 10 ** 9, storage=1)
+    running(srv, 2)
+    assert srv.stats()["peak_footprint"] <= held + bound
+    srv.close()
+    sound(cosm)
 
 
 def _weighted(n, m, wmax, seed):
