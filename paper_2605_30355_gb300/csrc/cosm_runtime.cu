@@ -2144,15 +2144,11 @@ static int batch_enqueue(cosm_batch *b, cudaStream_t st)
     return COSM_OK;
 }
 
-extern "C" int cosm_batch_run(cosm_batch *b, const int64_t *sweeps, const int32_t *replicas,
-                              const uint64_t *seeds, void *stream)
+// Lays a run out and launches it on the batch's stream, after earlier work on
+// the caller's and before later.
+static int batch_launch_run(cosm_batch *b, const int64_t *sweeps, const int32_t *replicas, const uint64_t *seeds,
+                            cudaStream_t user)
 {
-    NvtxRange range("cosm_batch_run");
-    if (!b || !sweeps || !replicas || !seeds) return fail(COSM_ERR_INVALID_ARG, "NULL argument");
-    for (size_t i = 0; i < b->hs.size(); ++i)
-        if (sweeps[i] < 1 || sweeps[i] >= ((int64_t)1 << 31) || replicas[i] < 1 || replicas[i] >= (1 << 24))
-            return fail(COSM_ERR_INVALID_ARG, "instance " + std::to_string(i) + ": bad sweeps or replicas");
-    cudaStream_t user = reinterpret_cast<cudaStream_t>(stream);
     cudaStream_t st = b->own;
     // order the batch after earlier work on the caller's stream
     cudaEvent_t e0;
@@ -2161,13 +2157,7 @@ extern "C" int cosm_batch_run(cosm_batch *b, const int64_t *sweeps, const int32_
     CK(cudaStreamWaitEvent(st, e0, 0));
     cudaEventDestroy(e0);
     int rc = batch_layout(b, sweeps, replicas, seeds, st);
-    if (rc) {
-        // some instances have a new layout: the last run's states and results end here
-        for (cosm_handle *h : b->hs) h->have_state = h->have_result = false;
-        b->have_result = false;
-        b->chosen.clear();
-        return rc;
-    }
+    if (rc) return rc;
     std::vector<int64_t> sig;
     sig.push_back((int64_t)(uintptr_t)b->d_insts.p);
     sig.push_back((int64_t)(uintptr_t)b->d_units.p);
@@ -2212,6 +2202,25 @@ extern "C" int cosm_batch_run(cosm_batch *b, const int64_t *sweeps, const int32_
     b->have_result = true;
     b->launches = (int64_t)b->classes.size() + 1;
     return COSM_OK;
+}
+
+extern "C" int cosm_batch_run(cosm_batch *b, const int64_t *sweeps, const int32_t *replicas,
+                              const uint64_t *seeds, void *stream)
+{
+    NvtxRange range("cosm_batch_run");
+    if (!b || !sweeps || !replicas || !seeds) return fail(COSM_ERR_INVALID_ARG, "NULL argument");
+    for (size_t i = 0; i < b->hs.size(); ++i)
+        if (sweeps[i] < 1 || sweeps[i] >= ((int64_t)1 << 31) || replicas[i] < 1 || replicas[i] >= (1 << 24))
+            return fail(COSM_ERR_INVALID_ARG, "instance " + std::to_string(i) + ": bad sweeps or replicas");
+    const int rc = batch_launch_run(b, sweeps, replicas, seeds, reinterpret_cast<cudaStream_t>(stream));
+    if (rc) {
+        // some instances may have a new layout: the last run's states and results
+        // end here
+        for (cosm_handle *h : b->hs) h->have_state = h->have_result = false;
+        b->have_result = false;
+        b->chosen.clear();
+    }
+    return rc;
 }
 
 extern "C" int cosm_batch_sync(cosm_batch *b)

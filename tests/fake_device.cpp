@@ -36,7 +36,7 @@ namespace {
 std::recursive_mutex mu;
 std::map<const char *, size_t> blocks;  // device allocations
 int64_t live = 0, peak = 0, fail_malloc = 0;
-std::atomic<int> fail_threads{0};
+std::atomic<int> fail_threads{0}, fail_graphs{0};
 std::atomic<int64_t> queries{0};  // of occupancies, since the last report
 bool pending = false;     // a legacy-stream copy or set that nothing has waited for
 uintptr_t next_handle = 0x1000;
@@ -338,6 +338,7 @@ cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t *g)
 }
 cudaError_t cudaGraphInstantiate(cudaGraphExec_t *e, cudaGraph_t, unsigned long long)
 {
+    if (fail_graphs > 0) return cudaErrorMemoryAllocation;
     *e = reinterpret_cast<cudaGraphExec_t>(0x30);
     return cudaSuccess;
 }
@@ -383,6 +384,7 @@ int cosm_probe_fp32(int32_t, double *, double *) { return COSM_ERR_CUDA; }
 // ---------------------------------------------------------------- the test's side
 void fake_fail_malloc(int64_t nth) { fail_malloc = nth; }  // the nth cudaMalloc from now on fails once
 void fake_fail_threads(int on) { fail_threads = on; }
+void fake_fail_graphs(int on) { fail_graphs = on; }
 int64_t fake_peak_bytes(void)  // since the last call
 {
     const int64_t p = peak;

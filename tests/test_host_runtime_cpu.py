@@ -190,6 +190,26 @@ def test_failed_batch_run_ends_the_batch_state(cosm):
     assert report(cosm)["bad"] == 0
 
 
+def test_failed_batch_launch_ends_the_batch_state(cosm):
+    # the layouts are new, the launch is not made: no state is read in them
+    b = cosm.Batch([g() for g in GRAPHS.values()])
+    b.run([20, 20], [4, 4], [1, 2])
+    cosm.lib().fake_fail_graphs(1)
+    with pytest.raises(cosm.CosmError) as err:
+        b.run([20, 20], [4096, 4096], [1, 2])
+    cosm.lib().fake_fail_graphs(0)
+    assert err.value.code == cosm.ERR_CUDA
+    b.replicas = [4, 4]
+    for call in (b.get_state, b.best, b.replica_cuts):
+        with pytest.raises(cosm.CosmError) as err:
+            call(0)
+        assert err.value.code == cosm.ERR_STATE
+    b.run([20, 20], [4, 4], [1, 2])
+    b.get_state(0)
+    b.close()
+    sound(cosm)
+
+
 def test_host_threads_that_cannot_be_created(fake_path):
     # the calling thread does the work; in a process of its own, as an escaping
     # exception would end it
